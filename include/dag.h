@@ -310,14 +310,16 @@ int dag_sssp_batched_u8(dag_plan* plan, dag_variant variant, int32_t delta, int3
  */
 int dag_plan_set_batched_graph(dag_plan* plan, int32_t on);
 /*
- * Kernel of the plan's batched synchronous and asynchronous solves with 32,
- * 64, 128 or 256 columns: on (1, when a plan is created) a warp owns all B
- * columns (B / 32 per lane, one vector access each) and an eighth of each
- * merge-path tile, so a source vertex's B values are gathered by one warp in
- * one burst; off (0), and always for other column counts and the delayed
- * form, each warp owns 32 columns and the CTA's warps walk every edge
- * together. Results agree within rounding (the same sweep; sums may be added
- * in another order). DAG_ERR_INVALID for a null plan.
+ * Kernel of the plan's batched synchronous and asynchronous solves: on (1,
+ * when a plan is created) the warps take runs of the merge path in turn, each
+ * over all B columns, so a source vertex's B values are read as one row; off
+ * (0), and always for the delayed form, each warp owns 32 columns and the
+ * CTA's warps walk every edge together. Results agree within rounding (the
+ * same sweep; sums may be added in another order). DAG_ERR_INVALID for a null
+ * plan. On, the plan keeps the runs' published partials (and for Bellman-Ford
+ * a byte per vertex), and, when B is not a multiple of 4 or the output array
+ * not 16-byte aligned, a state array of n rows of B values rounded up to a
+ * multiple of 4.
  */
 int dag_plan_set_batched_wide(dag_plan* plan, int32_t on);
 

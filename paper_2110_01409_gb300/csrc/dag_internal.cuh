@@ -192,6 +192,8 @@ struct dag_plan {
     size_t bx_bytes = 0;
     void* bsync = nullptr;
     size_t bsync_bytes = 0;
+    void* bruns = nullptr;      // runs: published partials and (Bellman-Ford) the vertices' last changes
+    size_t bruns_bytes = 0;
 };
 
 namespace dag {
@@ -244,6 +246,8 @@ int set_l1_carveout(const void* k, int device, int threads, size_t static_smem, 
 int get_warp_partition(dag_plan* plan, int W, int tile, Partition** out, cudaStream_t s);
 // The same over the merge path of rows [lo, hi) only (row-range sweeps).
 int get_warp_partition_range(dag_plan* plan, int W, int tile, int lo, int hi, Partition** out, cudaStream_t s);
+// Runs of the batched kernels (batched_runs.cu): cta_row / cta_tile hold each run's first row / in-edge.
+int get_batch_runs(dag_plan* plan, int W, int row_w, Partition** out, cudaStream_t s);
 int sweep_rows(dag_plan* plan, int mode, int lo, int hi, SweepParams& p, double* d_sums, cudaStream_t s);
 // sweep_warp.cu
 const void* sweep_warp_kernel_ptr(int mode, int variant, int ipt);

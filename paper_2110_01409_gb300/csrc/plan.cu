@@ -376,6 +376,42 @@ int get_warp_partition_range(dag_plan* plan, int W, int tile, int lo, int hi, Pa
     return DAG_OK;
 }
 
+// Runs of the batched kernels: run w of W starts at w / W of the merge path's
+// weight, a row's end weighing row_w and an in-edge 1 (a cut inside a row's end
+// goes before it). Rows [run_row[w], run_row[w + 1]) end in run w.
+__global__ void k_batch_runs(const int* rowptr, int n, long long total, int row_w, int W, int* run_row, int* run_nz)
+{
+    const int w = blockIdx.x * blockDim.x + threadIdx.x;
+    if (w > W) return;
+    const long long target = (long long)w * total / W;
+    int lo = 0, hi = n;  // first row whose end item ends past the target
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if ((long long)row_w * (mid + 1) + rowptr[mid + 1] > target) hi = mid;
+        else lo = mid + 1;
+    }
+    run_row[w] = lo;
+    run_nz[w] = lo == n ? rowptr[n] : (int)min(target - (long long)row_w * lo, (long long)rowptr[lo + 1]);
+}
+
+int get_batch_runs(dag_plan* plan, int W, int row_w, Partition** out, cudaStream_t s)
+{
+    const auto key = std::make_tuple(W, row_w, -1, -1);  // no row range has these bounds
+    auto it = plan->range_parts.find(key);
+    if (it != plan->range_parts.end()) { *out = &it->second; return DAG_OK; }
+    Partition part;
+    part.nblocks = W;
+    DAG_CUDA(dev_alloc(&part.cta_row, (W + 1) * sizeof(int)));
+    DAG_CUDA(dev_alloc(&part.cta_tile, (W + 1) * sizeof(int)));
+    k_batch_runs<<<(W + 1 + 255) / 256, 256, 0, s>>>(plan->rowptr, plan->n, (long long)row_w * plan->n + plan->m, row_w,
+                                                     W, part.cta_row, part.cta_tile);
+    DAG_CUDA(cudaGetLastError());
+    DAG_CUDA(cudaStreamSynchronize(s));  // ready for a later call on any stream
+    auto ins = plan->range_parts.emplace(key, part);
+    *out = &ins.first->second;
+    return DAG_OK;
+}
+
 // ---------------------------------------------------------------------------
 // Out-edge CSR: a stable radix sort of the in-edges by source keeps, within
 // each source, the in-CSR order, i.e. ascending targets.
@@ -733,6 +769,7 @@ extern "C" int dag_plan_destroy(dag_plan* p)
     dev_free(p->sync);
     cudaFree(p->bx);  // batched workspace: cudaMalloc (batched.cu)
     cudaFree(p->bsync);
+    dev_free(p->bruns);
     for (auto& kv : p->parts) {
         dev_free(kv.second.cta_row);
         dev_free(kv.second.cta_tile);

@@ -223,8 +223,8 @@ class Plan:
         _raise(lib().dag_plan_set_batched_graph(self.h, 1 if on else 0), False)
 
     def set_batched_wide(self, on: bool):
-        """Batched sync / async solves of 32, 64, 128 or 256 columns on the wide kernel (a warp per
-        share of a tile, all columns; on, the default) or on 32-column warps (off)."""
+        """Batched sync / async solves on runs of the merge path (a warp per run, all columns; on, the
+        default) or on 32-column warps (off)."""
         _raise(lib().dag_plan_set_batched_wide(self.h, 1 if on else 0), False)
 
     def set_warp_tile(self, items_per_lane: int):

@@ -218,3 +218,68 @@ def test_wide_batched_tiny_graphs(dag):
         for c in (0, 1, 5, 31):
             rstar = oracle.pagerank_fixed_point(g, 0.85, tele=V[:, c].astype(np.float64))
             assert np.abs(R[:, c] - rstar).sum() <= 1e-5, (variant, c)
+
+
+# ---- the run kernel (synchronous and asynchronous forms): any column count, rows spanning many warps' runs ----
+def _hub_graph():
+    """3,001 vertices: RMAT-like edges, two hubs whose in-edges span many runs, the last vertex among them, and a
+    tail of vertices without in-edges."""
+    rng = np.random.default_rng(5)
+    n, k = 3001, 12000
+    src = (rng.random(k) ** 3 * n).astype(np.int64)
+    dst = (rng.random(k) ** 2 * (n - 700)).astype(np.int64)
+    hubs = [np.stack([rng.permutation(n)[:2500], np.full(2500, h)]) for h in (17, n - 1)]
+    e = np.concatenate([np.stack([src, dst])] + hubs, axis=1)
+    e = np.unique(e[:, e[0] != e[1]], axis=1)
+    return I.from_edges(n, e[0], e[1])
+
+
+@pytest.mark.parametrize("B", [1, 2, 3, 6, 9, 20, 33, 72, 130, 300, 1024])
+@pytest.mark.parametrize("variant", ["sync", "async"])
+def test_runs_any_column_count(dag, B, variant):
+    # every lanes-per-row and chunks-per-lane shape, whole and ragged; outputs that are not 16-byte aligned go
+    # through the padded state; distances equal the oracle's, ranks lie within L1 1e-5 of the fixed point
+    g = _hub_graph()
+    plan = dag.Plan.from_graph(g, "cuda")
+    V = I.teleport_matrix(g.n, I.ppr_seed_sets(g.n, B, seed=3))
+    Vd = torch.from_numpy(V).cuda()
+    out = torch.empty(g.n * B + 1, dtype=torch.float32, device="cuda")[1:].view(g.n, B)
+    w = I.weights_u32(g, 9)
+    srcs = I.sources(g, B, seed=5) if B <= 300 else np.resize(I.sources(g, 300, seed=5), B)
+    sd = torch.from_numpy(srcs.view(np.int32)).cuda()
+    cols = sorted({0, B // 2, B - 1})
+    for o in (None, out):
+        R, iters, st = dag.ppr_batched(plan, Vd, 0.85, 1e-6, variant, 0, out=o)
+        assert st["converged"] and st["column_sweeps"] == int(iters.sum()) and st["sweeps"] == int(iters.max())
+        Rn = R.cpu().numpy().astype(np.float64)
+        for c in cols:
+            rstar = oracle.pagerank_fixed_point(g, 0.85, tele=V[:, c].astype(np.float64), tol=1e-12)
+            assert np.abs(Rn[:, c] - rstar).sum() <= 1e-5, c
+    for wd in (torch.from_numpy(w.astype(np.uint8)).cuda(), torch.from_numpy(w.view(np.int32)).cuda()):
+        D, iters, st = dag.sssp_batched(plan, sd, wd, variant, 0, out=torch.full((g.n * B + 1,), 7, dtype=torch.int32,
+                                                                                 device="cuda")[1:].view(g.n, B))
+        assert st["converged"]
+        Dn, its = D.cpu().numpy().view(np.uint32), iters.cpu().numpy()
+        for c in cols:
+            assert np.array_equal(Dn[:, c], oracle.dijkstra(g, w, int(srcs[c]))), c
+            if variant == "sync":
+                assert its[c] == oracle.sssp(g, w, int(srcs[c]), oracle.SYNC)[1]
+
+
+@pytest.mark.parametrize("variant", ["sync", "async"])
+def test_runs_long_path_and_sweep_limit(dag, variant):
+    # 600 sweeps: the last-change byte wraps twice; a solve stopped early reports its sweeps
+    n = 600
+    g = I.from_edges(n, np.arange(1, n), np.arange(n - 1))  # v <- v + 1: one hop per sweep against the row order
+    plan = dag.Plan.from_graph(g, "cuda")
+    w = torch.full((g.m,), 3, dtype=torch.uint8, device="cuda")
+    src = torch.tensor([n - 1, 300, n - 1], dtype=torch.int32, device="cuda")
+    D, iters, st = dag.sssp_batched(plan, src, w, variant, 0)
+    D = D.cpu().numpy().view(np.uint32)
+    for c, s in enumerate((n - 1, 300, n - 1)):
+        want = np.where(np.arange(n) <= s, 3 * (s - np.arange(n)), 0xFFFFFFFF).astype(np.uint32)
+        assert np.array_equal(D[:, c], want)
+    if variant == "sync":
+        assert iters.cpu().tolist() == [600, 301, 600]
+        _, _, st = dag.sssp_batched(plan, src, w, variant, 0, max_iters=5)
+        assert not st["converged"] and st["sweeps"] == 5
