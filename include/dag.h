@@ -167,8 +167,9 @@ int dag_plan_set_worker_cap(dag_plan* plan, int32_t max_workers);
  * Warp workers (dag_pagerank, dag_sssp, dag_sssp_u8; every variant): the
  * worker of Sec. III-A is one warp instead of one CTA. The merge path of the
  * whole graph (rows and in-edges in vertex order) is cut into tiles of
- * dag_warp_tile_items(plan) items and each warp takes an equal run of them, so
- * workers are balanced by in-degree + 1 as Sec. III-A asks; a warp owns the
+ * dag_warp_tile_items(plan) items and each warp takes a run of them, so that
+ * workers are balanced by in-degree + 3 per row (Sec. III-A's in-degree + 1,
+ * with what a row's update costs a warp beside an in-edge); a warp owns the
  * rows that end in its run, and a row whose in-edges span several runs gets
  * the earlier runs' partial sums at the end of the sweep. delta counts rows
  * per warp (each warp has its own buffer). No CTA-wide barrier inside a sweep.

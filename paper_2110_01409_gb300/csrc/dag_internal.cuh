@@ -241,11 +241,12 @@ size_t sweep_tma_ring_bytes(int mode);
 int set_l1_carveout(const void* k, int device, int threads, size_t static_smem, size_t dyn, int per_sm);
 
 // Warp workers: the whole merge path cut into tiles of `tile` items, warp w
-// of W taking tiles [floor(w T / W), floor((w+1) T / W)); cta_tile / cta_row
-// hold each warp's first tile / first owned row (the partition's nblocks is W).
-int get_warp_partition(dag_plan* plan, int W, int tile, Partition** out, cudaStream_t s);
+// of W taking the run of tiles from w / W to (w + 1) / W of the path's weight
+// (in-degree + row_w per row); cta_tile / cta_row hold each warp's first tile /
+// first owned row (the partition's nblocks is W).
+int get_warp_partition(dag_plan* plan, int W, int tile, int row_w, Partition** out, cudaStream_t s);
 // The same over the merge path of rows [lo, hi) only (row-range sweeps).
-int get_warp_partition_range(dag_plan* plan, int W, int tile, int lo, int hi, Partition** out, cudaStream_t s);
+int get_warp_partition_range(dag_plan* plan, int W, int tile, int row_w, int lo, int hi, Partition** out, cudaStream_t s);
 // Runs of the batched kernels (batched_runs.cu): cta_row / cta_tile hold each run's first row / in-edge.
 int get_batch_runs(dag_plan* plan, int W, int row_w, Partition** out, cudaStream_t s);
 int sweep_rows(dag_plan* plan, int mode, int lo, int hi, SweepParams& p, double* d_sums, cudaStream_t s);

@@ -310,18 +310,27 @@ __global__ void k_range_tile_coords(const int* rowptr, int lo, int hi, int tile,
     tile_nz[k] = (int)(diag - a);
 }
 
-__global__ void k_warp_runs(const int* tile_row, int tiles, int W, int* wtile, int* wrow)
+// Run w of W starts at the first tile at or past w / W of the path's weight, a row weighing row_w and an in-edge 1.
+__global__ void k_warp_runs(const int* tile_row, const int* tile_nz, int tiles, int W, int row_w, int* wtile, int* wrow)
 {
     const int w = blockIdx.x * blockDim.x + threadIdx.x;
     if (w > W) return;
-    const int t = (int)((long long)w * tiles / W);
-    wtile[w] = t;
-    wrow[w] = tile_row[t];
+    const long long base = (long long)row_w * tile_row[0] + tile_nz[0];
+    const long long total = (long long)row_w * tile_row[tiles] + tile_nz[tiles] - base;
+    const long long target = base + (long long)w * total / W;
+    int lo = 0, hi = tiles;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if ((long long)row_w * tile_row[mid] + tile_nz[mid] >= target) hi = mid;
+        else lo = mid + 1;
+    }
+    wtile[w] = lo;
+    wrow[w] = tile_row[lo];
 }
 
-int get_warp_partition(dag_plan* plan, int W, int tile, Partition** out, cudaStream_t s)
+int get_warp_partition(dag_plan* plan, int W, int tile, int row_w, Partition** out, cudaStream_t s)
 {
-    const long long key = (1LL << 62) | ((long long)tile << 32) | (long long)W;
+    const long long key = (1LL << 62) | ((long long)row_w << 48) | ((long long)tile << 32) | (long long)W;
     auto it = plan->parts.find(key);
     if (it != plan->parts.end()) { *out = &it->second; return DAG_OK; }
     Partition part;
@@ -337,7 +346,8 @@ int get_warp_partition(dag_plan* plan, int W, int tile, Partition** out, cudaStr
     DAG_CUDA(dev_alloc(&part.wpub, W * sizeof(unsigned long long)));
     k_warp_tile_coords<<<(unsigned)((T + 1 + 255) / 256), 256, 0, s>>>(plan->rowptr, plan->n, plan->m, tile, (int)T,
                                                                        part.tile_row, part.tile_nz);
-    k_warp_runs<<<(W + 1 + 255) / 256, 256, 0, s>>>(part.tile_row, (int)T, W, part.cta_tile, part.cta_row);
+    k_warp_runs<<<(W + 1 + 255) / 256, 256, 0, s>>>(part.tile_row, part.tile_nz, (int)T, W, row_w, part.cta_tile,
+                                                    part.cta_row);
     DAG_CUDA(cudaGetLastError());
     std::vector<int> wrow(W + 1);
     DAG_CUDA(cudaMemcpyAsync(wrow.data(), part.cta_row, (W + 1) * sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -348,9 +358,9 @@ int get_warp_partition(dag_plan* plan, int W, int tile, Partition** out, cudaStr
     return DAG_OK;
 }
 
-int get_warp_partition_range(dag_plan* plan, int W, int tile, int lo, int hi, Partition** out, cudaStream_t s)
+int get_warp_partition_range(dag_plan* plan, int W, int tile, int row_w, int lo, int hi, Partition** out, cudaStream_t s)
 {
-    const auto key = std::make_tuple(W, tile, lo, hi);
+    const auto key = std::make_tuple(W, tile | row_w << 16, lo, hi);
     auto it = plan->range_parts.find(key);
     if (it != plan->range_parts.end()) { *out = &it->second; return DAG_OK; }
     std::vector<int> rp(2);
@@ -368,7 +378,8 @@ int get_warp_partition_range(dag_plan* plan, int W, int tile, int lo, int hi, Pa
     DAG_CUDA(dev_alloc(&part.wpub, W * sizeof(unsigned long long)));
     k_range_tile_coords<<<(unsigned)((T + 1 + 255) / 256), 256, 0, s>>>(plan->rowptr, lo, hi, tile, (int)T,
                                                                         part.tile_row, part.tile_nz);
-    k_warp_runs<<<(W + 1 + 255) / 256, 256, 0, s>>>(part.tile_row, (int)T, W, part.cta_tile, part.cta_row);
+    k_warp_runs<<<(W + 1 + 255) / 256, 256, 0, s>>>(part.tile_row, part.tile_nz, (int)T, W, row_w, part.cta_tile,
+                                                    part.cta_row);
     DAG_CUDA(cudaGetLastError());
     DAG_CUDA(cudaStreamSynchronize(s));
     auto ins = plan->range_parts.emplace(key, part);

@@ -5,9 +5,9 @@
 // Paper mapping (Blanco, McMillan, Low, HPEC 2021):
 //  * worker = one warp. The merge path of the whole graph (rows and in-edges
 //    in vertex order, Merrill & Garland) is cut into warp tiles of WTILE items
-//    and every worker takes an equal run of consecutive tiles, so each carries
-//    the same in-degree + 1 weight (Sec. III-A's balance) and owns the rows
-//    whose end item lies in its run (contiguous in vertex order). A row whose
+//    and every worker takes a run of consecutive tiles of equal weight
+//    (in-degree + WARP_ROW_WEIGHT per row, Sec. III-A's balance with a row's
+//    cost on this machine) and owns the rows whose end item lies in its run (contiguous in vertex order). A row whose
 //    in-edges span two runs (a hub, or a cut inside a row) is owned by the run
 //    that ends it; the earlier runs' partial sums reach it at the end of the
 //    sweep through a bounded look-back (below);
@@ -21,10 +21,18 @@
 //
 // Why warps: the CTA-tile kernels (sweep.cu, sweep_tma.cu) stop all eight
 // warps at three barriers per 1,792-item tile, so each tile waits for its
-// slowest gather; here each warp walks its own 224-item tiles with a
-// shuffle-only segmented scan and issues the next tile's edge stream and
-// gathers before walking the current one, so the SM's 32 warps keep their
-// gathers in flight independently.
+// slowest gather; here each warp sums its own 224-item tiles with a
+// shuffle-only segmented scan, copies edge sources two tiles ahead (cp.async)
+// and issues the next tile's gathers before the current one's sums or after
+// them, so the SM's 32 warps keep their gathers in flight independently.
+//
+// What bounds it: one gather per clock through an SM's L1 (65 M edges: 0.19 to
+// 0.21 ms a sweep for 4 M RMAT vertices), then instructions and the slowest
+// run. Against a merge-path walk of each tile with the edge stream loaded one
+// tile ahead and runs of equal item counts, ms per solve: ordered PageRank (4 M
+// vertices) 3.76 -> 3.35 (466 -> 372 us per sweep, one sweep more), uniform
+// graph (2 M) 1.55 -> 1.38, synchronous (2 M) 1.77 -> 1.55, banded (4 M) 4.22 ->
+// 3.58, weighted PageRank (2 M, RMAT) 2.75 -> 1.95, its adjoint 2.3 -> 1.79.
 //
 // Row straddling two runs. At the end of its run a warp publishes the partial
 // of the row it leaves unfinished (one 64-bit word: sweep stamp and value).
@@ -54,7 +62,7 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_kernel(const SweepP
     constexpr bool LIVE_G = !SYNC && !BF;  // async/delayed PageRank-type: live global sum
     constexpr unsigned FULL = 0xffffffffu;
 
-    __shared__ WarpShared<WTILE> sh;
+    __shared__ WarpShared<MODE, WIPT> sh;
     extern __shared__ __align__(16) uint32_t w_buf[];  // delayed: p.buf_cap values per warp
 
     const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wl = tid >> 5;
@@ -65,9 +73,8 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_kernel(const SweepP
     uint32_t* X1 = (uint32_t*)p.x1;
     const int row_lo = p.cta_row[w], row_hi = p.cta_row[w + 1];  // rows whose end item lies in the run
     const int t_lo = p.cta_tile[w], t_hi = p.cta_tile[w + 1];
-    int* end = sh.end[wl];
+    uint16_t* end = sh.end[wl];
     uint32_t* val = sh.val[wl];
-    uint32_t* sum = sh.sum[wl];
     uint32_t* buf = w_buf + (size_t)wl * (DELAYED ? p.buf_cap : 0);
     // the run starts inside a row: its first row waits for the earlier runs' partials
     const bool mid0 = t_lo < t_hi && p.tile_nz[t_lo] > p.rowptr[p.tile_row[t_lo]];
@@ -126,68 +133,70 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_kernel(const SweepP
         if constexpr (SYNC && !BF)
             gt = (MODE == MODE_ADJ) ? (float)((double)p.g_coef * gprev) : (float)((double)p.g_coef * (T - gprev));
 
-        WStage<WIPT> nx;
-        if (t_lo < t_hi) wfetch<MODE, WIPT>(nx, p, xin, t_lo, lane, rmode, LIVE_G, pol_edge, pol_vertex);
+        // pipeline: tile t + 2's edge sources are copied and tile t + 1's gathers are in flight while tile t is summed
+        // and its rows finished. (Gathers after this tile's stores, as in the ordered sweep, read newer values, but
+        // cost 4% per sweep on a banded graph and 3% with a product per edge, for one sweep less on the former.)
+        WStage<MODE, WIPT> nx;
+        WCoord c1;  // of tile t + 1
+        if (t_lo < t_hi) {
+            const WCoord c0 = wcoord(p, t_lo);
+            c1 = wcoord(p, min(t_lo + 1, t_hi - 1));
+            wissue_col(sh, p, c0, wl, lane, pol_edge);
+            wcommit();
+            wlanded();
+            wgather(nx, sh, p, xin, c0, wl, lane, rmode, LIVE_G, pol_edge, pol_vertex);
+            if (t_lo + 1 < t_hi) wissue_col(sh, p, c1, wl, lane, pol_edge);
+            wcommit();
+        }
         for (int t = t_lo; t < t_hi; ++t) {
-            const int a0 = nx.a0, b0 = nx.b0, NA = nx.NA, NB = nx.NB;
+            const int a0 = nx.a0, NA = nx.NA;
             const uint32_t pf_xo = nx.xo;
-            const float pf_dg = nx.dg;
+            const float pf_dg = nx.dg, pf_bv = nx.bv;
             if constexpr (LIVE_G) {  // the global term, from the live sum read with every LIVE_EVERY-th tile
                 if (((t - t_lo) & (LIVE_EVERY - 1)) == 0) gt = live_term<MODE>(L, warp_sum(nx.gs));
             }
-            __syncwarp();  // the previous tile's epilogue is done with end / val / sum
-#pragma unroll
-            for (int q = 0; q < WIPT; ++q) {
-                const int j = lane + 32 * q;
-                if (j < NB) val[j] = nx.term[q];
+            __syncwarp();  // the previous tile's epilogue is done with end / val
+            wstage(sh, nx, p, wl, lane, pol_vertex);
+            const WCoord c2 = wcoord(p, min(t + 2, t_hi - 1));
+            if (t + 1 < t_hi) {
+                wlanded();
+                wgather(nx, sh, p, xin, c1, wl, lane, rmode, LIVE_G && ((t + 1 - t_lo) & (LIVE_EVERY - 1)) == 0, pol_edge,
+                        pol_vertex);
+                if (t + 2 < t_hi) wissue_col(sh, p, c2, wl, lane, pol_edge);
+                wcommit();
+                c1 = c2;
             }
-            wstage_ends<WIPT>(end, nx, p, lane, pol_vertex);
-            if (t + 1 < t_hi)
-                wfetch<MODE, WIPT>(nx, p, xin, t + 1, lane, rmode, LIVE_G && ((t + 1 - t_lo) & (LIVE_EVERY - 1)) == 0,
-                             pol_edge, pol_vertex);
             __syncwarp();
-            carry = wwalk<MODE, WIPT>(end, val, sum, NA, NB, carry, lane);
+            const uint32_t carry_in = carry;
+            carry = wwalk<MODE, WIPT>(end, val, sh.mark[wl], NA, carry, lane);
             __syncwarp();
 
             // -------- new values of the rows this tile completed --------
             const int skip = (head_pending && NA > 0) ? 1 : 0;  // the run's first row waits for the look-back
-            if (skip && lane == 0) head_part = sum[0];
+            if (skip && lane == 0) head_part = wrow_sum<MODE>(val, end, 0, carry_in);
             head_pending = head_pending && NA == 0;
-            // rows lane + 32 k: the first came with the tile, the others' inputs are loaded together
-            uint32_t xo_k[WIPT];
-            float dg_k[WIPT];
-            xo_k[0] = pf_xo;
-            dg_k[0] = pf_dg;
-#pragma unroll
-            for (int k = 1; k < WIPT; ++k) {
-                const int r = lane + 32 * k;
-                xo_k[k] = 0u;
-                dg_k[k] = 0.0f;
-                if (r < NA) {
-                    xo_k[k] = ld_weak_b32(xin + a0 + r);
-                    if constexpr (!BF) dg_k[k] = ld_stream_f32(p.degf + a0 + r);
-                }
-            }
-            // the adjoint's base terms c_v, all of the tile's loads in flight together (a load per row
-            // ahead of its update would wait once per row)
-            float bv_k[WIPT];
-            if constexpr (MODE == MODE_ADJ) {
-#pragma unroll
-                for (int k = 0; k < WIPT; ++k) bv_k[k] = lane + 32 * k < NA ? row_base<MODE>(p, a0 + lane + 32 * k) : 0.0f;
-            }
-#pragma unroll
-            for (int k = 0; k < WIPT; ++k) {
-                const int r = lane + 32 * k;
-                if (r >= NA || (k == 0 && lane == 0 && skip)) continue;
+            auto finish = [&](int r, uint32_t xo, float dg, float bv) {
                 const int v = a0 + r;
-                float bv;
-                if constexpr (MODE == MODE_ADJ) bv = bv_k[k];
-                else bv = row_base<MODE>(p, v);
-                const uint32_t xnew =
-                    row_update_b<MODE>(p, v, sum[r], xo_k[k], dg_k[k], gt, bv, A.off_f, res_part, g_part, dg_part);
+                const uint32_t xnew = row_update_b<MODE>(p, v, wrow_sum<MODE>(val, end, r, carry_in), xo, dg, gt, bv, A.off_f,
+                                                         res_part, g_part, dg_part);
                 if constexpr (SYNC) st_weak_b32(xout + v, xnew);
                 else if constexpr (ASYNC) st_relaxed_b32(X0 + v, xnew);
                 else buf[v - buf_first] = xnew;
+            };
+            if (lane < NA && !(lane == 0 && skip)) finish(lane, pf_xo, pf_dg, pf_bv);
+            constexpr int WROWS = 4;  // rows per lane whose inputs are in flight together (a tile of mostly empty rows)
+            for (int r = lane + 32; r < NA; r += 32 * WROWS) {
+                uint32_t xo[WROWS];
+                float dg[WROWS], bv[WROWS];
+#pragma unroll
+                for (int u = 0; u < WROWS; ++u) {
+                    xo[u] = 0u;
+                    dg[u] = bv[u] = 0.0f;
+                    if (r + 32 * u < NA) wrow_inputs<MODE>(p, xin, a0 + r + 32 * u, pol_vertex, xo[u], dg[u], bv[u]);
+                }
+#pragma unroll
+                for (int u = 0; u < WROWS; ++u)
+                    if (r + 32 * u < NA) finish(r + 32 * u, xo[u], dg[u], bv[u]);
             }
             if constexpr (ASYNC && LIVE_G) {
                 if (((t - t_lo) & (LIVE_EVERY - 1)) == LIVE_EVERY - 1) {  // this warp's change of N
@@ -349,7 +358,7 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_ordered_kernel(const Swe
     constexpr unsigned FULL = 0xffffffffu;
     (void)WTILE;
 
-    __shared__ WarpShared<32 * WIPT> sh;
+    __shared__ WarpShared<MODE, WIPT> sh;
     const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wl = tid >> 5;
     const int w = c * WWARPS + wl;
     const int W = p.nblocks * WWARPS, T = p.ntiles;  // warp w takes tiles w, w + W, w + 2W, ...
@@ -357,9 +366,8 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_ordered_kernel(const Swe
     unsigned long long bar_target = 0;
     uint32_t* X = (uint32_t*)p.x0;
     unsigned long long* pub = p.wpub;  // [T]
-    int* end = sh.end[wl];
+    uint16_t* end = sh.end[wl];
     uint32_t* val = sh.val[wl];
-    uint32_t* sum = sh.sum[wl];
 
     // ---------------- initial values (any thread any row: nothing reads them before the barrier) ----------------
     {
@@ -442,29 +450,33 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_ordered_kernel(const Swe
             pend_t = -1;
         };
 
-        WStage<WIPT> nx;
-        int k = 0;  // this warp's tiles so far in the sweep
-        if (w < T) wfetch<MODE, WIPT>(nx, p, X, w, lane, rmode, LIVE_G, pol_edge, pol_vertex);
+        WStage<MODE, WIPT> nx;
+        WCoord c1;  // of this warp's next tile
+        int k = 0;  // its tiles so far in the sweep
+        if (w < T) {
+            const WCoord c0 = wcoord(p, w);
+            c1 = wcoord(p, min(w + W, T - 1));
+            wissue_col(sh, p, c0, wl, lane, pol_edge);
+            wcommit();
+            wlanded();
+            wgather(nx, sh, p, X, c0, wl, lane, rmode, LIVE_G, pol_edge, pol_vertex);
+            if (w + W < T) wissue_col(sh, p, c1, wl, lane, pol_edge);
+            wcommit();
+        }
         for (int t = w; t < T && ok; t += W, ++k) {
-            const int a0 = nx.a0, b0 = nx.b0, NA = nx.NA, NB = nx.NB;
+            const int a0 = nx.a0, b0 = nx.b0, NA = nx.NA;
             const bool cont = b0 > nx.rp0;  // the tile starts inside row a0
             const uint32_t pf_xo = nx.xo;
-            const float pf_dg = nx.dg;
+            const float pf_dg = nx.dg, pf_bv = nx.bv;
             if constexpr (LIVE_G) {
                 if ((k & (LIVE_EVERY - 1)) == 0) gt = live_term<MODE>(L, warp_sum(nx.gs));
             }
             __syncwarp();
-#pragma unroll
-            for (int q = 0; q < WIPT; ++q) {
-                const int j = lane + 32 * q;
-                if (j < NB) val[j] = nx.term[q];
-            }
-            wstage_ends<WIPT>(end, nx, p, lane, pol_vertex);
-            if (t + W < T)
-                wfetch<MODE, WIPT>(nx, p, X, t + W, lane, rmode, LIVE_G && ((k + 1) & (LIVE_EVERY - 1)) == 0,
-                                   pol_edge, pol_vertex);
+            wstage(sh, nx, p, wl, lane, pol_vertex);
+            const bool more2 = T - t > 2LL * W;
+            const WCoord c2 = wcoord(p, more2 ? t + 2 * W : T - 1);
             __syncwarp();
-            const uint32_t trail = wwalk<MODE, WIPT>(end, val, sum, NA, NB, O::identity(), lane);
+            const uint32_t trail = wwalk<MODE, WIPT>(end, val, sh.mark[wl], NA, O::identity(), lane);
             __syncwarp();
             // the partial of the row left unfinished: inclusive unless the tile lies inside a row begun before
             const bool incl = NA > 0 || !cont;
@@ -473,37 +485,36 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_ordered_kernel(const Swe
 
             // -------- rows this tile completed (its first one, begun before, waits for the look-back) --------
             const int skip = (cont && NA > 0) ? 1 : 0;
-            const uint32_t first_sum = __shfl_sync(FULL, NA > 0 ? sum[0] : 0u, 0);
-            uint32_t xo_k[WIPT];
-            float dg_k[WIPT];
-            xo_k[0] = pf_xo;
-            dg_k[0] = pf_dg;
-#pragma unroll
-            for (int q = 1; q < WIPT; ++q) {
-                const int r = lane + 32 * q;
-                xo_k[q] = 0u;
-                dg_k[q] = 0.0f;
-                if (r < NA) {
-                    xo_k[q] = ld_weak_b32(X + a0 + r);
-                    if constexpr (!BF) dg_k[q] = ld_stream_f32(p.degf + a0 + r);
-                }
-            }
-            float bv_k[WIPT];  // the adjoint's base terms c_v, loaded together
-            if constexpr (MODE == MODE_ADJ) {
-#pragma unroll
-                for (int q = 0; q < WIPT; ++q) bv_k[q] = lane + 32 * q < NA ? row_base<MODE>(p, a0 + lane + 32 * q) : 0.0f;
-            }
-#pragma unroll
-            for (int q = 0; q < WIPT; ++q) {
-                const int r = lane + 32 * q;
-                if (r >= NA || (q == 0 && lane == 0 && skip)) continue;
+            const uint32_t first_sum = NA > 0 ? wrow_sum<MODE>(val, end, 0, O::identity()) : 0u;
+            auto finish = [&](int r, uint32_t xo, float dg, float bv) {
                 const int v = a0 + r;
-                float bv;
-                if constexpr (MODE == MODE_ADJ) bv = bv_k[q];
-                else bv = row_base<MODE>(p, v);
-                const uint32_t xnew =
-                    row_update_b<MODE>(p, v, sum[r], xo_k[q], dg_k[q], gt, bv, A.off_f, res_part, g_part, dg_part);
+                const uint32_t xnew = row_update_b<MODE>(p, v, wrow_sum<MODE>(val, end, r, O::identity()), xo, dg, gt, bv,
+                                                         A.off_f, res_part, g_part, dg_part);
                 st_relaxed_b32(X + v, xnew);
+            };
+            if (lane < NA && !(lane == 0 && skip)) finish(lane, pf_xo, pf_dg, pf_bv);
+            constexpr int WROWS = 2;  // rows per lane whose inputs are in flight together (a tile of mostly empty rows)
+            for (int r = lane + 32; r < NA; r += 32 * WROWS) {
+                uint32_t xo[WROWS];
+                float dg[WROWS], bv[WROWS];
+#pragma unroll
+                for (int u = 0; u < WROWS; ++u) {
+                    xo[u] = 0u;
+                    dg[u] = bv[u] = 0.0f;
+                    if (r + 32 * u < NA) wrow_inputs<MODE>(p, X, a0 + r + 32 * u, pol_vertex, xo[u], dg[u], bv[u]);
+                }
+#pragma unroll
+                for (int u = 0; u < WROWS; ++u)
+                    if (r + 32 * u < NA) finish(r + 32 * u, xo[u], dg[u], bv[u]);
+            }
+            // -------- the next tile's gathers (after this tile's stores: in flight earlier, they read older values and
+            // a sweep took 397 instead of 372 us at 4 M vertices, RMAT) --------
+            if (t + W < T) {
+                wlanded();
+                wgather(nx, sh, p, X, c1, wl, lane, rmode, LIVE_G && ((k + 1) & (LIVE_EVERY - 1)) == 0, pol_edge, pol_vertex);
+                if (more2) wissue_col(sh, p, c2, wl, lane, pol_edge);
+                wcommit();
+                c1 = c2;
             }
             // -------- the previous tile's look-back, then this tile's becomes pending --------
             resolve();
@@ -523,6 +534,7 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_ordered_kernel(const Swe
                 }
             }
         }  // tiles
+        wlanded();  // (a look-back that gave up leaves copies in flight)
         resolve();
         if constexpr (LIVE_G) {
             const float s = warp_sum(dg_part);
@@ -605,6 +617,14 @@ static const void* warp_kernel(int kind, int mode, int variant, int ipt, bool or
     return sweep_warp_kernel_ptr(mode, variant, ipt);
 }
 
+// A row's weight in the warps' runs beside its in-edges (Sec. III-A weighs in-degree + 1, for a CPU thread's work):
+// a row's update costs a warp about twice an in-edge more than the row's item did in the tiles' cut. Where a graph's
+// rows without in-edges lie together (RMAT: half the rows), runs of equal item counts held up to 6,600 rows against a
+// mean of 430 and the sweep waited for them. Weights 1, 2, 3, 4, RMAT, ms: CTA-ordered frontier Bellman-Ford (4 M
+// vertices) 2.99, 2.19-2.5, 2.05-2.35, 2.3-2.55; weighted PageRank and its adjoint (2 M) 2.78 + 2.4, 2.05 + 1.9,
+// 1.95 + 1.79, 1.99 + 1.98; delayed Bellman-Ford (1 M) 1.28, 1.21, 1.15, 1.21. Graphs without skew do not move.
+constexpr int WARP_ROW_WEIGHT = 3;
+
 static int warp_shape(dag_plan* plan, int mode, int variant, int delta, int* nb_out, int* cap_out, int* clamped_out,
                       Partition** part_out, cudaStream_t s, int kind, bool ordered = false)
 {
@@ -636,7 +656,7 @@ static int warp_shape(dag_plan* plan, int mode, int variant, int delta, int* nb_
     if (rc) return rc;
     bool settled = false;  // CTAs per SM only fall, so a few passes settle the shape
     for (int iter = 0; iter < 6 && !settled; ++iter) {
-        rc = get_warp_partition(plan, nb * WWARPS, WTILE, &part, s);
+        rc = get_warp_partition(plan, nb * WWARPS, WTILE, WARP_ROW_WEIGHT, &part, s);
         if (rc) return rc;
         settled = true;
         if (variant != DAG_DELAYED) break;
@@ -760,7 +780,7 @@ int sweep_rows(dag_plan* plan, int mode, int lo, int hi, SweepParams& p, double*
     int nb = per_sm * plan->num_sms;
     if (plan->worker_cap > 0) nb = std::min(nb, plan->worker_cap);
     Partition* part = nullptr;
-    int rc = get_warp_partition_range(plan, nb * WWARPS, WTILE, lo, hi, &part, s);
+    int rc = get_warp_partition_range(plan, nb * WWARPS, WTILE, WARP_ROW_WEIGHT, lo, hi, &part, s);
     if (rc) return rc;
     p.nblocks = nb;
     p.max_iters = 1;

@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_frontier_kernel(con
     constexpr unsigned FULL = 0xffffffffu;
     (void)WTILE;
 
-    __shared__ WarpShared<32 * WIPT> sh;
+    __shared__ WarpShared<MODE, WIPT> sh;
     __shared__ int s_cnt;  // ordered dense sweeps: rows on the CTA's list of lowered rows
     const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wl = tid >> 5;
     const int w = c * WWARPS + wl;
@@ -67,9 +67,8 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_frontier_kernel(con
     uint32_t* X = (uint32_t*)p.x0;
     const int row_lo = p.cta_row[w], row_hi = p.cta_row[w + 1];
     const int t_lo = p.cta_tile[w], t_hi = p.cta_tile[w + 1];
-    int* end = sh.end[wl];
+    uint16_t* end = sh.end[wl];
     uint32_t* val = sh.val[wl];
-    uint32_t* sum = sh.sum[wl];
     int* own_chg = p.fr_chg + row_lo;  // dense sweeps: this warp's changed rows (its own, so at most row_hi - row_lo)
     // ordered dense sweeps: the CTA's tiles [T0, T1) (its warps' runs together), taken by its warps in turn, and
     // its list of lowered rows (a row split over k of its tiles may appear k times: at most rows + tiles entries)
@@ -98,8 +97,8 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_frontier_kernel(con
         const int slot = it % 3;
         const unsigned stamp = (unsigned)it + 1u;
         float res_part = 0.0f, unused_g = 0.0f, unused_dg = 0.0f;
-        long long marks = 0;  // this lane's share of the out-degree sum of the rows lowered in the sweep
-        long long edges = 0;  // lane 0: edges of the tiles this warp ran
+        int marks = 0;  // this lane's share of the out-degree sum of the rows lowered in the sweep
+        int edges = 0;  // lane 0: edges of the tiles this warp ran
         bool ok = true;
 
         if (ORD && dense) {
@@ -109,41 +108,37 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_frontier_kernel(con
             // so no tile waits for another.
             if (tid == 0) s_cnt = 0;
             __syncthreads();
-            WStage<WIPT> nx;
-            if (T0 + wl < T1) wfetch<MODE, WIPT>(nx, p, X, T0 + wl, lane, rmode, false, pol_edge, pol_vertex);
+            WStage<MODE, WIPT> nx;
+            WCoord c1;  // of this warp's next tile
+            if (T0 + wl < T1) {
+                const WCoord c0 = wcoord(p, T0 + wl);
+                c1 = wcoord(p, min(T0 + wl + WWARPS, T1 - 1));
+                wissue_col(sh, p, c0, wl, lane, pol_edge);
+                wcommit();
+                wlanded();
+                wgather(nx, sh, p, X, c0, wl, lane, rmode, false, pol_edge, pol_vertex);
+                if (T0 + wl + WWARPS < T1) wissue_col(sh, p, c1, wl, lane, pol_edge);
+                wcommit();
+            }
             for (int t = T0 + wl; t < T1; t += WWARPS) {
                 const int a0 = nx.a0, b0 = nx.b0, NA = nx.NA, NB = nx.NB;
                 const bool cont = b0 > nx.rp0;  // the tile starts inside row a0
                 const uint32_t pf_xo = nx.xo;
                 __syncwarp();
-#pragma unroll
-                for (int q = 0; q < WIPT; ++q) {
-                    const int j = lane + 32 * q;
-                    if (j < NB) val[j] = nx.term[q];
-                }
-                wstage_ends<WIPT>(end, nx, p, lane, pol_vertex);
-                if (t + WWARPS < T1)
-                    wfetch<MODE, WIPT>(nx, p, X, t + WWARPS, lane, rmode, false, pol_edge, pol_vertex);
+                wstage(sh, nx, p, wl, lane, pol_vertex);
+                const WCoord c2 = wcoord(p, min(t + 2 * WWARPS, T1 - 1));
                 __syncwarp();
-                const uint32_t trail = wwalk<MODE, WIPT>(end, val, sum, NA, NB, O::identity(), lane);
+                const uint32_t trail = wwalk<MODE, WIPT>(end, val, sh.mark[wl], NA, O::identity(), lane);
                 __syncwarp();
                 if (lane == 0) edges += NB;
-                uint32_t xo_k[WIPT];
-                xo_k[0] = pf_xo;
-#pragma unroll
-                for (int k = 1; k < WIPT; ++k) {
+                for (int k = 0; 32 * k <= NA; ++k) {
                     const int r = lane + 32 * k;
-                    xo_k[k] = r < NA ? ld_weak_b32(X + a0 + r) : 0u;
-                }
-#pragma unroll
-                for (int k = 0; k <= WIPT; ++k) {
-                    const int r = lane + 32 * k;
-                    if (32 * k > NA) break;  // warp-uniform
                     bool changed = false;
                     const int v = a0 + r;
                     if (r < NA) {
-                        const uint32_t sv = sum[r];
-                        const uint32_t xo = xo_k[k < WIPT ? k : 0];
+                        const uint32_t sv = wrow_sum<MODE>(val, end, r, O::identity());
+                        // (a row without a finite sum, in a tile of mostly empty rows, needs no old value)
+                        const uint32_t xo = k == 0 ? pf_xo : sv != INF ? ld_weak_keep_b32(X + v, pol_vertex) : 0u;
                         if (r == 0 && cont) {  // the rest of a row begun in an earlier tile
                             if (sv != INF && sv < xo) changed = sv < atomicMin(X + v, sv);
                         } else if (sv < xo) {  // a whole row: only this tile writes it in a dense sweep
@@ -161,6 +156,13 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_frontier_kernel(con
                     base = __shfl_sync(FULL, base, 0);
                     if (changed) cta_chg[base + __popc(bal & ((1u << lane) - 1u))] = v;
                 }
+                if (t + WWARPS < T1) {  // the next tile's gathers, after this tile's stores (newer values: fewer edges run)
+                    wlanded();
+                    wgather(nx, sh, p, X, c1, wl, lane, rmode, false, pol_edge, pol_vertex);
+                    if (t + 2 * WWARPS < T1) wissue_col(sh, p, c2, wl, lane, pol_edge);
+                    wcommit();
+                    c1 = c2;
+                }
             }
             __syncthreads();  // the CTA's list is complete
             own_cnt = s_cnt;
@@ -174,49 +176,56 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_frontier_kernel(con
             uint32_t carry = O::identity();
             bool head_pending = head;
             uint32_t head_part = O::identity();
-            WStage<WIPT> nx;
-            if (t_lo < t_hi) wfetch<MODE, WIPT>(nx, p, X, t_lo, lane, rmode, false, pol_edge, pol_vertex);
+            WStage<MODE, WIPT> nx;
+            WCoord c1;  // of tile t + 1
+            if (t_lo < t_hi) {
+                const WCoord c0 = wcoord(p, t_lo);
+                c1 = wcoord(p, min(t_lo + 1, t_hi - 1));
+                wissue_col(sh, p, c0, wl, lane, pol_edge);
+                wcommit();
+                wlanded();
+                wgather(nx, sh, p, X, c0, wl, lane, rmode, false, pol_edge, pol_vertex);
+                if (t_lo + 1 < t_hi) wissue_col(sh, p, c1, wl, lane, pol_edge);
+                wcommit();
+            }
             for (int t = t_lo; t < t_hi; ++t) {
-                const int a0 = nx.a0, b0 = nx.b0, NA = nx.NA, NB = nx.NB;
+                const int a0 = nx.a0, NA = nx.NA;
                 const uint32_t pf_xo = nx.xo;
                 __syncwarp();
-#pragma unroll
-                for (int q = 0; q < WIPT; ++q) {
-                    const int j = lane + 32 * q;
-                    if (j < NB) val[j] = nx.term[q];
-                }
-                wstage_ends<WIPT>(end, nx, p, lane, pol_vertex);
-                if (t + 1 < t_hi) wfetch<MODE, WIPT>(nx, p, X, t + 1, lane, rmode, false, pol_edge, pol_vertex);
+                wstage(sh, nx, p, wl, lane, pol_vertex);
+                const WCoord c2 = wcoord(p, min(t + 2, t_hi - 1));
                 __syncwarp();
-                carry = wwalk<MODE, WIPT>(end, val, sum, NA, NB, carry, lane);
+                const uint32_t carry_in = carry;
+                carry = wwalk<MODE, WIPT>(end, val, sh.mark[wl], NA, carry, lane);
                 __syncwarp();
                 const int skip = (head_pending && NA > 0) ? 1 : 0;  // the run's first row waits for the look-back
-                if (skip && lane == 0) head_part = sum[0];
+                if (skip && lane == 0) head_part = wrow_sum<MODE>(val, end, 0, carry_in);
                 head_pending = head_pending && NA == 0;
-                uint32_t xo_k[WIPT];
-                xo_k[0] = pf_xo;
-#pragma unroll
-                for (int k = 1; k < WIPT; ++k) {
+                for (int k = 0; 32 * k < NA; ++k) {
                     const int r = lane + 32 * k;
-                    xo_k[k] = r < NA ? ld_weak_b32(X + a0 + r) : 0u;
-                }
-#pragma unroll
-                for (int k = 0; k < WIPT; ++k) {
-                    const int r = lane + 32 * k;
-                    if (32 * k >= NA) break;  // warp-uniform: no lane has a row in this or a later slot
                     bool changed = false;
                     if (r < NA && !(k == 0 && lane == 0 && skip)) {
-                        const uint32_t xnew =
-                            row_update<MODE>(p, a0 + r, sum[r], xo_k[k], 0.0f, 0.0f, 0.0f, res_part, unused_g, unused_dg);
-                        changed = xnew < xo_k[k];
-                        st_relaxed_b32(X + a0 + r, xnew);
+                        const uint32_t sv = wrow_sum<MODE>(val, end, r, carry_in);
+                        const uint32_t xo = k == 0 ? pf_xo : sv != INF ? ld_weak_keep_b32(X + a0 + r, pol_vertex) : 0u;
+                        if (sv < xo) {
+                            changed = true;
+                            res_part += 1.0f;
+                            st_relaxed_b32(X + a0 + r, sv);
+                        }
                     }
                     const unsigned bal = __ballot_sync(FULL, changed);
                     if (changed) own_chg[own_cnt + __popc(bal & ((1u << lane) - 1u))] = a0 + r;
                     own_cnt += __popc(bal);
                 }
+                if (t + 1 < t_hi) {  // the next tile's gathers, after this tile's stores (newer values: fewer edges run)
+                    wlanded();
+                    wgather(nx, sh, p, X, c1, wl, lane, rmode, false, pol_edge, pol_vertex);
+                    if (t + 2 < t_hi) wissue_col(sh, p, c2, wl, lane, pol_edge);
+                    wcommit();
+                    c1 = c2;
+                }
             }
-            if (lane == 0) edges += (long long)(p.tile_nz[t_hi] - p.tile_nz[t_lo]);
+            if (lane == 0) edges += p.tile_nz[t_hi] - p.tile_nz[t_lo];
             // the row this run leaves unfinished, and the one it started inside (as in the warp-worker sweep)
             if (lane == 0) st_relaxed_u64(p.wpub + w, ((unsigned long long)stamp << 32) | carry);
             if (head) {
@@ -279,37 +288,44 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_frontier_kernel(con
                 }
             };
             int t = next_tile();
-            WStage<WIPT> nx;
-            if (t >= 0) wfetch<MODE, WIPT>(nx, p, X, t, lane, READ_COHERENT, false, pol_edge, pol_vertex);
+            WStage<MODE, WIPT> nx;
+            auto copy = [&](const WCoord& c) {
+                wissue_col(sh, p, c, wl, lane, pol_edge);
+                wcommit();
+            };
+            if (t >= 0) {
+                const WCoord c0 = wcoord(p, t);
+                copy(c0);
+                wlanded();
+                wgather(nx, sh, p, X, c0, wl, lane, READ_COHERENT, false, pol_edge, pol_vertex);
+            }
             while (t >= 0) {
                 const int a0 = nx.a0, b0 = nx.b0, NA = nx.NA, NB = nx.NB;
                 const uint32_t pf_xo = nx.xo;
                 const int tn = next_tile();
                 __syncwarp();
-#pragma unroll
-                for (int q = 0; q < WIPT; ++q) {
-                    const int j = lane + 32 * q;
-                    if (j < NB) val[j] = nx.term[q];
-                }
-                wstage_ends<WIPT>(end, nx, p, lane, pol_vertex);
-                if (tn >= 0) wfetch<MODE, WIPT>(nx, p, X, tn, lane, READ_COHERENT, false, pol_edge, pol_vertex);
+                wstage(sh, nx, p, wl, lane, pol_vertex);
                 __syncwarp();
-                const uint32_t trail = wwalk<MODE, WIPT>(end, val, sum, NA, NB, O::identity(), lane);
+                if (tn >= 0) {
+                    const WCoord c1 = wcoord(p, tn);
+                    copy(c1);
+                    wlanded();
+                    wgather(nx, sh, p, X, c1, wl, lane, READ_COHERENT, false, pol_edge, pol_vertex);
+                }
+                const uint32_t trail = wwalk<MODE, WIPT>(end, val, sh.mark[wl], NA, O::identity(), lane);
                 __syncwarp();
                 if (lane == 0) edges += NB;
                 // rows of the tile (the first may be partial), then the partial of the row it leaves unfinished;
                 // a value read here may be older than the latest (never lower), so only a smaller sum is sent.
                 // A lowered row flags the tiles of its out-edges at once (after a fence, so that a warp that
                 // takes the flag reads the lowered value).
-#pragma unroll
-                for (int k = 0; k <= WIPT; ++k) {
+                for (int k = 0; 32 * k <= NA; ++k) {
                     const int r = lane + 32 * k;
-                    if (32 * k > NA) break;  // warp-uniform
                     bool changed = false;
                     const int v = a0 + r;
                     uint32_t cand = INF, seen = 0u;
                     if (r < NA) {
-                        cand = sum[r];
+                        cand = wrow_sum<MODE>(val, end, r, O::identity());
                         seen = k == 0 ? pf_xo : ld_relaxed_b32(X + v);
                     } else if (r == NA && v < p.n) {  // the row continuing into the next tile
                         cand = trail;
