@@ -62,12 +62,11 @@ struct Stage {
     long long gs;        // one stripe of the live global sum (warp 0)
 };
 
-// Issues the coalesced loads of tile t (everything except the gathers).
+// Issues the coalesced loads of tile t that do not depend on the state (edge stream, row ends).
 template <int MODE>
-__device__ __forceinline__ void stage_issue(Stage<MODE>& st, const SweepParams& p, const uint32_t* xin, int t, int tid,
-                                            bool weak, uint64_t pol_edge, uint64_t pol_vertex)
+__device__ __forceinline__ void stage_issue(Stage<MODE>& st, const SweepParams& p, int t, int tid, uint64_t pol_edge,
+                                            uint64_t pol_vertex)
 {
-    constexpr bool BF = MODE == MODE_BF || MODE == MODE_BF8;
     st.a0 = p.tile_row[t];
     st.b0 = p.tile_nz[t];
     st.NA = p.tile_row[t + 1] - st.a0;
@@ -89,6 +88,14 @@ __device__ __forceinline__ void stage_issue(Stage<MODE>& st, const SweepParams& 
         const int i = tid + q * NT;
         st.rend[q] = (i < st.NA) ? (int)ld_vertex_b32(p.rowptr + st.a0 + i + 1, pol_vertex) - st.b0 : 0;
     }
+}
+
+// Issues the loads of its first rows' old values and out-degrees.
+template <int MODE>
+__device__ __forceinline__ void stage_rows(Stage<MODE>& st, const SweepParams& p, const uint32_t* xin, int tid, bool weak,
+                                           uint64_t pol_vertex)
+{
+    constexpr bool BF = MODE == MODE_BF || MODE == MODE_BF8;
 #pragma unroll
     for (int k = 0; k < RP; ++k) {
         const int r = tid + k * NT;
@@ -235,7 +242,8 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_kernel(const SweepParams 
         // and its gathers too (issued before barrier C of t).
         Stage<MODE> nx;
         if (ntl > 0) {
-            stage_issue<MODE>(nx, p, xin, tile_at(0), tid, weak, pol_edge, pol_vertex);
+            stage_issue<MODE>(nx, p, tile_at(0), tid, pol_edge, pol_vertex);
+            stage_rows<MODE>(nx, p, xin, tid, weak, pol_vertex);
             stage_gather<MODE>(nx, xin, tid, weak, pol_vertex, s_buf, 0, 0);
             if constexpr (LIVE_G) {
                 if (warp == 0) nx.gs = ld_relaxed_i64(&sb->stripe[lane * GSTRIDE]);
@@ -300,7 +308,10 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_kernel(const SweepParams 
                 t_prev = t;
                 if (tid == 0) edges_done += NB;
             }
-            if (more) stage_issue<MODE>(nx, p, xin, tile_at(i + 1), tid, weak, pol_edge, pol_vertex);
+            if (more) {
+                stage_issue<MODE>(nx, p, tile_at(i + 1), tid, pol_edge, pol_vertex);
+                stage_rows<MODE>(nx, p, xin, tid, weak, pol_vertex);
+            }
             float gt = gterm;
             if constexpr (LIVE_G) {
                 gt = sh.gt;
@@ -358,13 +369,11 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_kernel(const SweepParams 
             __syncthreads();  // the CTA's list of changed rows is complete
             marks += changed_marks(p.fr_chg + row_lo, sh.nchg, p.fr_orow);
         }
-        double res_d = (double)res_part, g_d = FRONTIER ? (double)marks : (double)g_part;  // marks: exact in FP64
+        if constexpr (FRONTIER) block_add_count(sh, res_part, &sb->acc_res[slot], marks, &sb->acc_g[slot]);
+        else block_add(sh, res_part, &sb->acc_res[slot], g_part, ((SYNC && !BF) || MODE == MODE_ADJ) ? &sb->acc_g[slot] : nullptr);
         marks = 0;
-        block_sum2(sh, res_d, g_d);
-        if (tid == 0) {
-            if (res_d != 0.0) atomicAdd(&sb->acc_res[slot], res_d);
-            if ((FRONTIER || (SYNC && !BF) || MODE == MODE_ADJ) && g_d != 0.0) atomicAdd(&sb->acc_g[slot], g_d);
-            if (FRONTIER && edges_done) atomicAdd((unsigned long long*)&sb->edges, (unsigned long long)edges_done);
+        if (FRONTIER && tid == 0) {
+            if (edges_done) atomicAdd((unsigned long long*)&sb->edges, (unsigned long long)edges_done);
             edges_done = 0;
         }
         if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns)) return;
@@ -517,6 +526,15 @@ int settle_shape(dag_plan* plan, int mode, int variant, int delta,
     int nb = 0;
     int rc = max_workers(plan, mode, variant, 0, &nb);
     if (rc) return rc;
+    {
+        // A small graph's sweep is its grid barrier: one CTA per tile (two at least, so that a barrier has someone to
+        // wait for). Above half the resident CTAs the SMs are better filled evenly (banded, 60 K vertices: 568 CTAs of
+        // a tile each 447 us, 608 of a little less 424).
+        const int cap = delayed_row_cap(variant, delta);
+        const long long row_w = cap > 0 ? (TILE + cap - 1) / cap : 1;
+        const long long tiles = std::max(2LL, (row_w * plan->n + plan->m + TILE - 1) / TILE);
+        if (2 * tiles <= nb) nb = (int)tiles;
+    }
     if (plan->worker_cap > 0 && nb > plan->worker_cap) nb = plan->worker_cap;
     int cap = 0, clamped = 0;
     long long max_cap = 0;  // largest buffer (values) one CTA can hold beside its static shared memory

@@ -65,6 +65,8 @@ struct SweepShared {
     double gprev;                        // broadcast of the previous sweep's global sum
     double T;                            // broadcast of the teleport total / ||c||_1
     alignas(8) unsigned long long fill_bar[RING];  // staging-ring mbarriers (TMA kernel)
+    // the threads' sums of a sweep (block_add): val is free once the last tile's walk is behind a barrier
+    __device__ __forceinline__ float& part(int k, int w, int l) { return ((float*)val)[k * NT + 32 * w + l]; }
 };
 
 // Block sum of two doubles; the result is valid in thread 0.
@@ -81,6 +83,45 @@ __device__ __forceinline__ void block_sum2(SH& sh, double& a, double& b)
         for (int k = 0; k < NWARP; ++k) { a += sh.red0[k]; b += sh.red1[k]; }
     }
     __syncthreads();
+}
+
+// Adds the CTA's sums of the threads' FP32 parts a, and with db b, to *da and *db in FP64 (no atomic for a zero sum).
+// FP64 issues at 2 lanes per clock and SM: a shuffle sum in every warp took 2.6 us of an SM's FP64 pipe at the end of
+// every sweep; here one warp per sum adds the parts from shared memory. The caller's next __syncthreads (the grid
+// barrier's) orders the atomics before what follows. A call, not inlined: inlined it cost the delayed sweeps up to 250
+// bytes of spills in their tile loops.
+template <class SH>
+__device__ __noinline__ void block_add(SH& sh, float a, double* da, float b = 0.0f, double* db = nullptr)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    sh.part(0, warp, lane) = a;
+    if (db) sh.part(1, warp, lane) = b;
+    __syncthreads();
+    if (warp == 0 || (warp == 1 && db)) {
+        double s0 = 0.0, s1 = 0.0;
+#pragma unroll 1
+        for (int k = 0; k < NWARP; k += 2) {
+            s0 += (double)sh.part(warp, k, lane);
+            s1 += (double)sh.part(warp, k + 1, lane);
+        }
+        const double t = warp_sum(s0 + s1);
+        if (lane == 0 && t != 0.0) atomicAdd(warp == 0 ? da : db, t);
+    }
+}
+
+// block_add of a and, as an exact count, of c (frontier sweeps: tile marks).
+template <class SH>
+__device__ __forceinline__ void block_add_count(SH& sh, float a, double* da, long long c, double* dc)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    c = warp_sum(c);
+    if (lane == 0) sh.red0[warp] = (double)c;  // (exact)
+    block_add(sh, a, da);
+    if (threadIdx.x == NT - 1) {
+        double t = 0.0;
+        for (int k = 0; k < NWARP; ++k) t += sh.red0[k];
+        if (t != 0.0) atomicAdd(dc, t);
+    }
 }
 
 // A thread's part of one tile's merge path (Merrill & Garland): IPT items from

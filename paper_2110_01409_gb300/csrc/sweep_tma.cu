@@ -480,13 +480,10 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_tma_kernel(const SweepPar
                 marks += changed_marks(p.fr_chg + row_lo, sh.nchg, p.fr_orow);
             }
         }
-        double res_d = (double)res_part, g_d = FRONTIER ? (double)marks : (double)g_part;  // marks: exact in FP64
+        if constexpr (FRONTIER) block_add_count(sh, res_part, &sb->acc_res[slot], (long long)marks, &sb->acc_g[slot]);
+        else block_add(sh, res_part, &sb->acc_res[slot], g_part, MODE == MODE_ADJ ? &sb->acc_g[slot] : nullptr);
         marks = 0;
-        block_sum2(sh, res_d, g_d);
-        if (tid == 0 && res_d != 0.0) atomicAdd(&sb->acc_res[slot], res_d);
-        if (MODE == MODE_ADJ && tid == 0 && g_d != 0.0) atomicAdd(&sb->acc_g[slot], g_d);
         if (FRONTIER && tid == 0) {
-            if (g_d != 0.0) atomicAdd(&sb->acc_g[slot], g_d);
             // edges of the tiles run: an own sweep runs all of the CTA's tiles
             const int e = shared ? edges_done : p.tile_nz[tile_hi] - p.tile_nz[tile_lo];
             if (e) atomicAdd((unsigned long long*)&sb->edges, (unsigned long long)e);

@@ -266,12 +266,8 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_kernel(const SweepP
         }
 
         // -------- end of sweep: residual, barrier, stopping rule --------
-        double res_d = (double)res_part, g_d = (double)g_part;
-        block_sum2(sh, res_d, g_d);
-        if (tid == 0) {
-            if (res_d != 0.0) atomicAdd(&sb->acc_res[slot], res_d);
-            if ((SYNC || MODE == MODE_ADJ) && !BF && g_d != 0.0) atomicAdd(&sb->acc_g[slot], g_d);
-        }
+        __syncwarp();  // (block_add uses the warp's val)
+        block_add(sh, res_part, &sb->acc_res[slot], g_part, ((SYNC || MODE == MODE_ADJ) && !BF) ? &sb->acc_g[slot] : nullptr);
         if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns)) return;
         if (tid == 0) {
             sh.res = ld_relaxed_f64(&sb->acc_res[slot]);
@@ -382,7 +378,7 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_ordered_kernel(const Swe
         }
     }
     if (p.skip_barrier_cta0 && c == 0) return;  // test hook: the others' waits must run out
-    if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns)) return;
+    if (!grid_barrier_call(sb, p.nblocks, bar_target, p.timeout_ns)) return;
 
     double T_tot = 1.0;
     if (tid == 0 && !BF) {
@@ -543,11 +539,9 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_ordered_kernel(const Swe
         }
 
         // -------- end of sweep: residual, barrier, stopping rule --------
-        double res_d = (double)res_part, g_d = (double)g_part;
-        block_sum2(sh, res_d, g_d);
-        if (tid == 0 && res_d != 0.0) atomicAdd(&sb->acc_res[slot], res_d);
-        if (MODE == MODE_ADJ && tid == 0 && g_d != 0.0) atomicAdd(&sb->acc_g[slot], g_d);
-        if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns)) return;
+        __syncwarp();  // (block_add uses the warp's val)
+        block_add(sh, res_part, &sb->acc_res[slot], g_part, MODE == MODE_ADJ ? &sb->acc_g[slot] : nullptr);
+        if (!grid_barrier_call(sb, p.nblocks, bar_target, p.timeout_ns)) return;
         if (tid == 0) {
             sh.res = ld_relaxed_f64(&sb->acc_res[slot]);
             if (MODE == MODE_ADJ) sh.gprev = ld_relaxed_f64(&sb->acc_g[slot]);
@@ -648,6 +642,10 @@ static int warp_shape(dag_plan* plan, int mode, int variant, int delta, int* nb_
         const int rc = set_l1_carveout(k, plan->device, NT, fa.sharedSizeBytes, dyn, per_sm);
         if (rc) return rc;
         int n_cta = per_sm * plan->num_sms;
+        // a small graph's sweep is its grid barrier: one tile per warp (two CTAs at least), as settle_shape; 5,000
+        // vertices in 608 CTAs took 545 us, the runs' look-back waiting along runs without a tile, in 34 112
+        const long long tiles = ((long long)plan->n + plan->m + WTILE - 1) / WTILE;
+        n_cta = (int)std::min((long long)n_cta, std::max(2LL, (tiles + WWARPS - 1) / WWARPS));
         if (plan->worker_cap > 0) n_cta = std::min(n_cta, plan->worker_cap);  // the cap counts CTAs
         *out = n_cta;
         return DAG_OK;

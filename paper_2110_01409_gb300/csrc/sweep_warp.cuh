@@ -20,6 +20,11 @@ constexpr int WMINBLOCKS = 4;        // CTAs per SM the register budget is sized
 constexpr int LIVE_EVERY = 8;        // async / delayed PageRank: a warp reads and adds to the live sum every 8
                                      // tiles (1,792 items, the CTA-tile kernels' tile), not every tile
 
+// A tile's merge-path coordinates: rows [a0, a1) end in it, edges [b0, b1).
+struct WCoord {
+    int a0, b0, a1, b1;
+};
+
 template <int MODE, int WIPT>
 struct WarpShared {
     static constexpr int WTILE = 32 * WIPT;
@@ -30,11 +35,8 @@ struct WarpShared {
     double red0[NWARP];
     double red1[NWARP];
     double res, gprev, T;
-};
-
-// A tile's merge-path coordinates: rows [a0, a1) end in it, edges [b0, b1).
-struct WCoord {
-    int a0, b0, a1, b1;
+    // a warp's own val, which it is done with at the end of its tiles
+    __device__ __forceinline__ float& part(int k, int w, int l) { return ((float*)val[w])[32 * k + l]; }
 };
 
 __device__ __forceinline__ WCoord wcoord(const SweepParams& p, int t)
@@ -230,12 +232,6 @@ __device__ __forceinline__ uint32_t wwalk(const uint16_t* end, uint32_t* val, ui
     return __shfl_sync(0xffffffffu, sv, 31);
 }
 
-__device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p)
-{
-    unsigned long long v;
-    asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
 __device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned long long v)
 {
     asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(v) : "memory");

@@ -355,13 +355,9 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_frontier_kernel(con
         }
 
         // ---------------- end of sweep: rows lowered, marks, edges; barrier; stopping rule ----------------
-        double res_d = (double)res_part, g_d = (double)marks;  // marks: exact in FP64
-        block_sum2(sh, res_d, g_d);
+        __syncwarp();  // (block_add uses the warp's val)
+        block_add_count(sh, res_part, &sb->acc_res[slot], (long long)marks, &sb->acc_g[slot]);
         if (lane == 0 && edges) atomicAdd((unsigned long long*)&sb->edges, (unsigned long long)edges);
-        if (tid == 0) {
-            if (res_d != 0.0) atomicAdd(&sb->acc_res[slot], res_d);
-            if (g_d != 0.0) atomicAdd(&sb->acc_g[slot], g_d);
-        }
         if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns)) return;
         if (tid == 0) {
             sh.res = ld_relaxed_f64(&sb->acc_res[slot]);
@@ -383,7 +379,8 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_frontier_kernel(con
             break;
         }
         const bool was_dense = dense;
-        dense = sh.gprev > sparse_marks;
+        // (with fr_sparse 0 every sweep is dense, also one after lowering only rows without out-edges)
+        dense = sh.gprev > sparse_marks || p.fr_sparse <= 0.0f;
         if (!dense && was_dense) {
             // into the sparse phase: the rows the dense sweep lowered flag the tiles of their out-edges (a sparse
             // sweep's lowered rows flagged theirs as they went)
