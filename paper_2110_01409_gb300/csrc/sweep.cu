@@ -30,13 +30,13 @@
 //
 // Per tile: all loads (edge stream, gathers, row ends, the rows' old values)
 // are issued in one staging phase into registers; after barrier (A) each
-// thread walks its IPT items of the merge path; after barrier (B) each thread
-// takes the carry of a row begun by earlier threads from a block segmented
-// prefix over the warps' run totals and finishes the rows it ends. A delayed
-// flush is copied out between (A) and (B) of the following tile, so it costs
-// no barrier. This kernel keeps its shared memory small (about 22 KB per CTA
-// plus the delay buffer) because its gathers of the previous iterate or of the
-// SM's view of the live array are ordinary loads that live off L1 hits.
+// thread adds its IPT edges and closes rows at their marked ends; after barrier
+// (B) each thread reads its rows' sums, with the carry of a row begun by earlier
+// warps, and updates them. A delayed flush is copied out between (A) and (B) of
+// the following tile, so it costs no barrier. This kernel keeps its shared
+// memory small (about 18 KB per CTA plus the delay buffer) because its gathers of
+// the previous iterate or of the SM's view of the live array are ordinary loads
+// that live off L1 hits.
 #include <algorithm>
 #include <climits>
 #include <cstdint>
@@ -48,6 +48,7 @@
 namespace dag {
 
 constexpr int RP = 2;  // epilogue rows per thread whose inputs are loaded with the tile
+static_assert(RP == 2, "the epilogue takes the second from pf_x[RP - 1]");
 
 // Registers of a tile being loaded ahead of use.
 template <int MODE>
@@ -121,7 +122,7 @@ __device__ __forceinline__ void stage_gather(Stage<MODE>& st, const uint32_t* xi
 #pragma unroll
     for (int q = 0; q < IPT; ++q) {
         const int j = tid + q * NT;
-        uint32_t term = 0u;
+        uint32_t term = Op<MODE>::identity();
         if (j < st.NB) {
             const unsigned off = (unsigned)(st.col[q] - lbase);
             const uint32_t xv = off < (unsigned)lcnt ? lbuf[off]
@@ -150,7 +151,7 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_kernel(const SweepParams 
     constexpr bool DELAYED = VAR == DAG_DELAYED;
     constexpr bool LIVE_G = !SYNC && !BF;  // async/delayed PageRank-type: live global sum
 
-    __shared__ SweepShared<true> sh;
+    __shared__ SweepShared sh;
     extern __shared__ uint32_t s_buf[];  // delay buffer (DELAYED)
 
     const int c = blockIdx.x;
@@ -204,6 +205,10 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_kernel(const SweepParams 
     long long marks = 0;       // frontier: out-degree sum of this thread's changed rows in the sweep
     bool dense = true;         // frontier: this sweep runs every tile
     if (tid == 0) sh.nchg = 0;
+    clear_marks(sh, 0);
+    clear_marks(sh, 1);
+    __syncthreads();
+    int buf = 0;  // the tile's buffer of terms and marks
     int it = 0;
     bool converged = false;
     double last_res = 0.0;
@@ -214,7 +219,7 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_kernel(const SweepParams 
         uint32_t* xout = SYNC ? ((it & 1) ? X0 : X1) : X0;
         // per-thread partial sums in FP32 (few rows each); FP64 from the block reduction on
         float res_part = 0.0f, g_part = 0.0f, dg_part = 0.0f;
-        uint32_t carry = O::identity();  // thread 0: partial of the row continuing into the next tile
+        uint32_t carry = O::identity();  // partial of the row continuing into the next tile
         bool flush_pending = false;      // delayed: the buffer is copied out during the next tile's walk
         float gterm = 0.0f;
         if constexpr (SYNC && !BF) {
@@ -257,14 +262,17 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_kernel(const SweepParams 
             const int NA = real ? nx.NA : 0, NB = real ? nx.NB : 0;
             uint32_t pf_x[RP];
             float pf_d[RP];
+            int pf_e = 0, pf_b = 0;  // end of row tid, and of the row before it (lane 0; the others' is a neighbour's)
             // -------- tile t into shared memory --------
             if (real) {
 #pragma unroll
                 for (int q = 0; q < IPT; ++q) {
                     const int jj = tid + q * NT;
-                    if (jj < NB) sh.val[jj] = nx.term[q];
-                    if (jj < NA) sh.rowend[jj] = nx.rend[q];
+                    sh.val[buf][jj] = nx.term[q];  // (identity past the last edge)
+                    if (jj < NA) mark_row_end(sh, buf, nx.rend[q]);
                 }
+                pf_e = nx.rend[0];
+                if (lane == 0 && tid < NA) pf_b = tid > 0 ? (int)ld_vertex_b32(p.rowptr + a0 + tid, pol_vertex) - b0 : 0;
 #pragma unroll
                 for (int k = 0; k < RP; ++k) { pf_x[k] = nx.pfx[k]; pf_d[k] = nx.pfd[k]; }
                 if constexpr (LIVE_G) {
@@ -274,8 +282,7 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_kernel(const SweepParams 
                     }
                 }
             }
-            if (tid == 0) sh.rowend[NA] = INT_MAX;
-            __syncthreads();  // (A) tile staged; every thread is done with the previous tile
+            __syncthreads();  // (A) tile staged; every thread is done with the previous tile's rows
 
             // -------- delayed: copy out the buffer filled by the previous tiles --------
             if constexpr (DELAYED) {
@@ -304,7 +311,7 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_kernel(const SweepParams 
             const bool more = i + 1 < ntl;
             if constexpr (FRONTIER) {
                 const int t = tile_at(i);
-                if (tid == 0 && t != t_prev + 1) carry = O::identity();  // the row before was not run
+                if (t != t_prev + 1) carry = O::identity();  // the row before was not run
                 t_prev = t;
                 if (tid == 0) edges_done += NB;
             }
@@ -318,32 +325,39 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_kernel(const SweepParams 
                 if (warp == 0 && more) nx.gs = ld_relaxed_i64(&sb->stripe[lane * GSTRIDE]);
             }
 
-            // -------- merge-path walk over this thread's IPT items, block segmented scan --------
-            const WalkOut w = walk_tile<MODE, true>(sh, [&](int i) { return sh.rowend[i]; }, NA, NB, carry);
-            __syncthreads();  // (B) warp run totals visible
-            const uint32_t E_last = finish_scan<MODE>(sh, w);
-            if (tid == 0) carry = E_last;  // partial of row NA for the next tile
+            // -------- row sums --------
+            const uint32_t row0 = carry;  // (thread 0) the first row's, when it ended before the tile's first edge
+            walk_tile<MODE>(sh, buf, (NA > 0 && pf_e == 0) ? O::identity() : carry);
+            __syncthreads();  // (B) row sums and the warps' partials visible
+            const uint32_t E = row_sums<MODE>(sh);
+            carry = __shfl_sync(0xffffffffu, E, NWARP - 1);  // partial of row NA for the next tile
             if (more)
                 stage_gather<MODE>(nx, xin, tid, weak, pol_vertex, s_buf, buf_first,
                                    (DELAYED && p.local_read) ? buf_cnt : 0);
-            __syncthreads();  // (C) row sums final
+            clear_marks(sh, buf);
 
             // -------- epilogue: new values of the rows this tile completed --------
-#pragma unroll
-            for (int k = 0; k < IPT; ++k) {
+            for (int k = 0; k * NT + 32 * warp < NA; ++k) {  // warp-uniform
                 const int r = tid + k * NT;
-                if (r >= NA) break;
                 const int v = a0 + r;
-                const uint32_t sum = sh.rowsum[r];
-                uint32_t xo_bits;
+                uint32_t xo_bits = 0u;
                 float dg = 0.0f;
+                int e = pf_e, eb = pf_b;
                 if (k < RP) {
-                    xo_bits = pf_x[k < RP ? k : 0];
-                    dg = pf_d[k < RP ? k : 0];
-                } else {
-                    xo_bits = weak ? ld_weak_b32(xin + v) : ld_relaxed_b32(xin + v);
-                    if constexpr (!BF) dg = ld_stream_f32(p.degf + v);
+                    xo_bits = k == 0 ? pf_x[0] : pf_x[RP - 1];
+                    dg = k == 0 ? pf_d[0] : pf_d[RP - 1];
                 }
+                if (k > 0 && r < NA) {
+                    e = (int)ld_vertex_b32(p.rowptr + v + 1, pol_vertex) - b0;
+                    if (lane == 0) eb = (int)ld_vertex_b32(p.rowptr + v, pol_vertex) - b0;
+                    if (k >= RP) {
+                        xo_bits = weak ? ld_weak_b32(xin + v) : ld_relaxed_b32(xin + v);
+                        if constexpr (!BF) dg = ld_stream_f32(p.degf + v);
+                    }
+                }
+                const int ep = __shfl_up_sync(0xffffffffu, e, 1);
+                const uint32_t sum = row_sum<MODE>(sh, buf, E, e, lane > 0 ? ep : eb, r == 0 ? row0 : O::identity());
+                if (r >= NA) continue;
                 const uint32_t xnew = row_update<MODE>(p, v, sum, xo_bits, dg, gt, A.off_f, res_part, g_part, dg_part);
                 if constexpr (FRONTIER)  // the row goes on the CTA's list; its marks are counted at the sweep's end
                     log_changed(p.fr_chg + row_lo, &sh.nchg, xnew < xo_bits, v, epilogue_lanes(NA, k));
@@ -351,6 +365,7 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_kernel(const SweepParams 
                 else if constexpr (DELAYED) s_buf[v - buf_first] = xnew;
                 else st_relaxed_b32(xout + v, xnew);
             }
+            buf ^= 1;
             if constexpr (DELAYED) {
                 buf_cnt += NA;
                 // flush at delta, at the block end, or (buffer clamped to what fits) when the next tile might not fit

@@ -1,8 +1,8 @@
 // Device pieces shared by the two sweep kernels (sweep.cu: register-staged
 // tiles, used by the synchronous and delayed forms; sweep_tma.cu: TMA-staged
 // tiles, used by the asynchronous form): the per-mode reduction, the
-// Bellman-Ford relaxation, block reductions, the merge-path walk of one tile
-// with its block segmented scan, and the row update of PageRank (Sec. IV-A),
+// Bellman-Ford relaxation, block reductions, the row sums of one tile, and the
+// row update of PageRank (Sec. IV-A),
 // its adjoint and Bellman-Ford.
 #pragma once
 
@@ -43,16 +43,13 @@ __device__ __forceinline__ uint32_t relax(uint32_t du, uint32_t w)
     return (s < du || s == INF) ? INF - 1u : s;
 }
 
-// Shared memory of one sweep CTA. ROWEND: the tile's row ends live here (the
-// register-staged kernel); the TMA kernel reads them from its staging ring.
-template <bool ROWEND>
+// Shared memory of one sweep CTA. Edge terms and marks are double-buffered, so
+// that a tile is staged while slower threads finish the rows of the one before.
 struct SweepShared {
-    uint32_t val[TILE];                  // edge terms of the tile
-    int rowend[ROWEND ? TILE + 1 : 1];   // tile-relative row end offsets (+ sentinel)
-    uint32_t rowsum[TILE];               // per-row reduction of the tile
-    int wkey[NWARP];                     // row in progress after each warp's last lane
-    int wfirst[NWARP];                   // row in progress after each warp's first lane
-    uint32_t wval[NWARP];                // warp-local inclusive run total at the last lane
+    uint32_t val[2][TILE];               // edge terms of the tile, then row sums at each row's last edge (walk_tile)
+    uint32_t mark[2][TILE / 4 + 4];      // byte j: edge j is the last of its row
+    int wpos[NWARP];                     // the first row end among each warp's edges (-1: none)
+    uint32_t wtail[NWARP];               // each warp's sum after its last row end
     double red0[NWARP];
     double red1[NWARP];
     float gt;                            // the tile's global (dangling) term from the live sum
@@ -124,102 +121,95 @@ __device__ __forceinline__ void block_add_count(SH& sh, float a, double* da, lon
     }
 }
 
-// A thread's part of one tile's merge path (Merrill & Garland): IPT items from
-// diagonal tid * IPT, rows 0..NA-1 and edges 0..NB-1 of the tile, row ends from
-// rowend(i) (tile-relative, i < NA; with SENTINEL, rowend(NA) is INT_MAX too,
-// which saves a compare per step). Rows it ends get their partial in
-// sh.rowsum; the row in progress after its last item is (key, sv) after the
-// warp-level segmented scan, whose warp summaries go to sh.wkey / wval / wfirst.
-// The caller places barrier (B) after this.
-struct WalkOut {
-    int i_start;  // first row this thread touches
-    int key;      // row in progress after its last item
-    uint32_t sv;  // warp-inclusive run total of that row
-    bool emitted; // it ended at least one row
-};
+// Marks the row end e (tile-relative; 0: before the tile's first edge) in a tile being staged. Rows without edges
+// mark the end of the row before them again.
+template <class SH>
+__device__ __forceinline__ void mark_row_end(SH& sh, int buf, int e)
+{
+    if (e > 0) ((uint8_t*)sh.mark[buf])[e - 1] = 1;
+}
+template <class SH>
+__device__ __forceinline__ void clear_marks(SH& sh, int buf)
+{
+    for (int i = threadIdx.x; i < TILE / 4 + 4; i += NT) sh.mark[buf][i] = 0u;
+}
 
-template <int MODE, bool SENTINEL, class SH, class RE>
-__device__ __forceinline__ WalkOut walk_tile(SH& sh, const RE& rowend, int NA, int NB, uint32_t carry)
+// The row sums of one staged tile, left in val at each row's last edge: thread t adds edges t IPT .. + IPT - 1 and
+// closes a row where its mark is set; a shuffle segmented scan joins the rows that span lanes; rows that span warps
+// are joined when they are read (row_sums, row_sum). carry (thread 0): the partial of the row continuing from the
+// previous tile, unless that row ended before this tile's first edge. The caller places a barrier after this; with
+// the one after staging these are the tile's two barriers. (A merge-path walk over rows and edges, with its own row
+// sum array, needed three, and its two kinds of steps diverged.)
+template <int MODE, class SH>
+__device__ __forceinline__ void walk_tile(SH& sh, int buf, uint32_t carry)
 {
     using O = Op<MODE>;
+    static_assert(IPT == 7, "a thread's marks are read as two words");
+    constexpr unsigned FULL = 0xffffffffu;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int L = NA + NB;
-    const int k0 = min(tid * IPT, L);
-    int lo = max(0, k0 - NB), hi = min(k0, NA);
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (rowend(mid) <= k0 - 1 - mid) lo = mid + 1;
-        else hi = mid;
-    }
-    WalkOut w;
-    int i = lo, j = k0 - lo;
-    w.i_start = i;
-    w.emitted = false;
-    uint32_t acc = (tid == 0) ? carry : O::identity();
-    int re = (SENTINEL || i < NA) ? rowend(i) : INT_MAX;
+    uint32_t* val = sh.val[buf] + tid * IPT;
+    const uint32_t* mk = sh.mark[buf] + ((tid * IPT) >> 2);
+    const int sft = 8 * ((tid * IPT) & 3);
+    const uint32_t w1 = mk[1];
+    const uint32_t m0 = __funnelshift_r(mk[0], w1, sft), m1 = __funnelshift_r(w1, mk[2], sft);
+    int first = -1;
+    uint32_t acc = tid == 0 ? carry : O::identity();
 #pragma unroll
     for (int q = 0; q < IPT; ++q) {
-        if (k0 + q < L) {
-            if (re <= j) {
-                sh.rowsum[i] = acc;
-                w.emitted = true;
-                acc = O::identity();
-                ++i;
-                re = (SENTINEL || i < NA) ? rowend(i) : INT_MAX;
-            } else {
-                acc = O::combine(acc, sh.val[j]);
-                ++j;
-            }
+        acc = O::combine(acc, val[q]);
+        if (((q < 4 ? m0 : m1) >> (8 * (q & 3))) & 1u) {
+            val[q] = acc;
+            acc = O::identity();
+            if (first < 0) first = q;
         }
     }
-    // segmented scan of (row in progress, partial) within the warp
-    w.key = i;
+    const unsigned closing = __ballot_sync(FULL, first >= 0);
+    const unsigned closed = closing & (FULL >> (31 - lane));
+    const int from = closed ? 31 - __clz(closed) : 0;
     uint32_t sv = acc;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t ov = __shfl_up_sync(0xffffffffu, sv, o);
-        const int ok = __shfl_up_sync(0xffffffffu, w.key, o);
-        if (lane >= o && ok == w.key) sv = O::combine(sv, ov);
+        const uint32_t ov = __shfl_up_sync(FULL, sv, o);
+        if (lane - o >= from) sv = O::combine(sv, ov);
     }
-    w.sv = sv;
-    if (lane == 31) { sh.wkey[warp] = w.key; sh.wval[warp] = sv; }
-    if (lane == 0) sh.wfirst[warp] = w.key;
-    return w;
+    const uint32_t cin = __shfl_up_sync(FULL, sv, 1);
+    if (lane > 0 && first >= 0) val[first] = O::combine(val[first], cin);
+    if (lane == 31) sh.wtail[warp] = sv;
+    if (closing ? lane == __ffs(closing) - 1 : lane == 0) sh.wpos[warp] = closing ? tid * IPT + first : -1;
 }
 
-// After barrier (B): the carry of a row begun by earlier threads, from a
-// segmented scan over the warps' run totals (in every warp), added to the
-// first row this thread ended. Returns the partial of the row that continues
-// into the next tile (the same value in every thread).
+// After the barrier that follows walk_tile, in every warp: lane w < NWARP gets the partial, over all the warps up to
+// w, of the row in progress after warp w's edges (lane NWARP - 1: of the row that continues into the next tile).
 template <int MODE, class SH>
-__device__ __forceinline__ uint32_t finish_scan(SH& sh, const WalkOut& w)
+__device__ __forceinline__ uint32_t row_sums(const SH& sh)
 {
     using O = Op<MODE>;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    uint32_t E;  // run total ending at warp w's last lane, over all earlier warps
-    {
-        const int wl = lane < NWARP ? lane : NWARP - 1;
-        const int wk = sh.wkey[wl];
-        const bool head = lane == 0 || sh.wfirst[wl] != wk || sh.wkey[wl > 0 ? wl - 1 : 0] != wk;
-        E = sh.wval[wl];
-        int hd = head ? 1 : 0;
+    const int lane = threadIdx.x & 31, wl = lane < NWARP ? lane : NWARP - 1;
+    uint32_t E = sh.wtail[wl];
+    bool head = lane == 0 || sh.wpos[wl] >= 0;
 #pragma unroll
-        for (int o = 1; o < NWARP; o <<= 1) {
-            const uint32_t oe = __shfl_up_sync(0xffffffffu, E, o);
-            const int oh = __shfl_up_sync(0xffffffffu, hd, o);
-            if (lane >= o && !hd) E = O::combine(E, oe);
-            if (lane >= o) hd |= oh;
+    for (int o = 1; o < NWARP; o <<= 1) {
+        const uint32_t oe = __shfl_up_sync(0xffffffffu, E, o);
+        const int oh = __shfl_up_sync(0xffffffffu, head ? 1 : 0, o);
+        if (lane >= o && !head) {
+            E = O::combine(E, oe);
+            head = oh != 0;
         }
     }
-    const uint32_t E_prev = __shfl_sync(0xffffffffu, E, warp > 0 ? warp - 1 : 0);
-    const int key_prev = warp > 0 ? sh.wkey[warp - 1] : -1;
-    const int k_first = __shfl_sync(0xffffffffu, w.key, 0);
-    const uint32_t pre = (warp > 0 && key_prev == k_first) ? E_prev : O::identity();
-    const uint32_t S = (w.key == k_first) ? O::combine(w.sv, pre) : w.sv;
-    uint32_t cin = __shfl_up_sync(0xffffffffu, S, 1);
-    if (lane == 0) cin = (warp > 0) ? E_prev : O::identity();
-    if (tid > 0 && w.emitted) sh.rowsum[w.i_start] = O::combine(sh.rowsum[w.i_start], cin);
-    return __shfl_sync(0xffffffffu, E, NWARP - 1);  // whole warp takes part
+    return E;
+}
+
+// The sum of the row whose edges end at e and began at b (tile-relative, the previous row's end) from E of row_sums;
+// `none` for a row without edges in the tile. Every lane of the warp calls it.
+template <int MODE, class SH>
+__device__ __forceinline__ uint32_t row_sum(const SH& sh, int buf, uint32_t E, int e, int b, uint32_t none)
+{
+    using O = Op<MODE>;
+    const int w = e > 0 ? (e - 1) / (32 * IPT) : 0;
+    const uint32_t c = __shfl_sync(0xffffffffu, E, w > 0 ? w - 1 : 0);
+    if (e <= b) return none;
+    const uint32_t s = sh.val[buf][e - 1];
+    return (w > 0 && sh.wpos[w] == e - 1) ? O::combine(s, c) : s;
 }
 
 // ---------------------------------------------------------------------------

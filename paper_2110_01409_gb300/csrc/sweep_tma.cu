@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_tma_kernel(const SweepPar
     static_assert(!FRONTIER || BF, "frontier: Bellman-Ford only");
     constexpr bool LIVE_G = !BF;  // PageRank-type: live global sum
 
-    __shared__ SweepShared<false> sh;
+    __shared__ SweepShared sh;
     extern __shared__ __align__(128) unsigned char ring[];  // tile staging ring
 
     const int c = blockIdx.x;
@@ -240,6 +240,9 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_tma_kernel(const SweepPar
         sh.nchg = 0;
         for (int k = 0; k < NWARP; ++k) sh.dgw[k] = 0.0f;
     }
+    clear_marks(sh, 0);
+    clear_marks(sh, 1);
+    int buf = 0;  // the tile's buffer of terms and marks
 
     // ---------------- initial values (a grid-stride pass, init_values) ----------------
     {
@@ -353,8 +356,9 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_tma_kernel(const SweepPar
 #pragma unroll
                 for (int k = 0; k < IPT; ++k) {
                     const int jj = tid + k * NT;
-                    if (jj < NB) sh.val[jj] = edge_term<MODE>(term[k], aux, ao + jj);
+                    sh.val[buf][jj] = jj < NB ? edge_term<MODE>(term[k], aux, ao + jj) : Op<MODE>::identity();
                 }
+                for (int i = tid; i < NA; i += NT) mark_row_end(sh, buf, rend[i] - b0);
                 if constexpr (LIVE_G) {
                     if (warp == 0) {  // the tile's global term, formed once
                         const long long G = warp_sum(gs);
@@ -362,16 +366,16 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_tma_kernel(const SweepPar
                     }
                 }
             }
-            __syncthreads();  // (A) tile staged; every thread is done with the previous tile
+            __syncthreads();  // (A) tile staged; every thread is done with the previous tile's rows
             if constexpr (LIVE_G) flush_dg(sh, sb, c, L.S);  // the previous tile's change of N, one atomic per CTA
 
             const int t1 = sh.tq[(q + 1) % RING];  // the next tile (known since the previous tile)
             const bool more = t1 >= 0;
             const float gt = LIVE_G ? sh.gt : 0.0f;
             if constexpr (FRONTIER) {
-                if (tid == 0 && shared) {
+                if (shared) {
                     carry = Op<MODE>::identity();  // a claimed tile starts afresh
-                    edges_done += NB;
+                    if (tid == 0) edges_done += NB;
                 }
             }
             // -------- the copies of the tile after next, the next tile's gathers --------
@@ -397,9 +401,10 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_tma_kernel(const SweepPar
                 }
             }
 
-            // -------- merge-path walk over this thread's IPT items, block segmented scan --------
-            const WalkOut w = walk_tile<MODE, false>(sh, [&](int i) { return rend[i] - b0; }, NA, NB, carry);
-            __syncthreads();  // (B) warp run totals visible; sh.tq of the tile after next written
+            // -------- row sums --------
+            const uint32_t row0 = carry;  // the first row's, when it ended before the tile's first edge
+            walk_tile<MODE>(sh, buf, (NA > 0 && rend[0] == b0) ? Op<MODE>::identity() : carry);
+            __syncthreads();  // (B) row sums and the warps' partials visible; sh.tq of the tile after next written
             if (sh.abort) {   // a staging wait ran out (error recorded): drain own copies, leave
                 if (tid == 0) {
                     if (more) (void)mbar_wait(&sh.fill_bar[(q + 1) % RING], ((q + 1) / RING) & 1u, p.timeout_ns);
@@ -408,11 +413,12 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_tma_kernel(const SweepPar
                 }
                 return;  // the other CTAs' barrier waits end on the recorded error
             }
-            const uint32_t E_last = finish_scan<MODE>(sh, w);
-            if (tid == 0) {
-                if (!shared) {
-                    carry = E_last;  // partial of row NA for the next tile
-                } else if constexpr (FRONTIER) {
+            const uint32_t E = row_sums<MODE>(sh);
+            const uint32_t E_last = __shfl_sync(0xffffffffu, E, NWARP - 1);
+            clear_marks(sh, buf);
+            if (!shared) carry = E_last;  // partial of row NA for the next tile
+            if constexpr (FRONTIER) {
+                if (tid == 0 && shared) {
                     if (E_last != Op<MODE>::identity()) {  // the row continuing into another tile: relax it now
                         const int v = a0 + NA;
                         const uint32_t old = atomicMin(X + v, E_last);
@@ -424,19 +430,32 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_tma_kernel(const SweepPar
                     }
                 }
             }
-            __syncthreads();  // (C) row sums final
 
             // -------- epilogue: new values of the rows this tile completed --------
             const uint32_t* old = (const uint32_t*)(ring + R::OFF_OLD) + (q % RING) * R::OLD_INTS + g.old_off();
             const uint32_t* degs = (const uint32_t*)(ring + R::OFF_DEG) + (q % RING) * R::DEG_INTS + g.old_off();
-#pragma unroll
-            for (int k = 0; k < IPT; ++k) {
+            // the first NT rows' inputs came with the tile; the others' (a tile of mostly empty rows) are loaded one
+            // turn ahead
+            uint32_t xo_next = 0u;
+            float dg_next = 0.0f;
+            if (tid < NA) {
+                xo_next = old[tid];
+                if constexpr (!BF) dg_next = __uint_as_float(degs[tid]);
+            }
+            for (int k = 0; k * NT + 32 * warp < NA; ++k) {  // warp-uniform
                 const int r = tid + k * NT;
-                if (r >= NA) break;
                 const int v = a0 + r;
+                const uint32_t xo_bits = xo_next;
+                const float dg = dg_next;
+                if (r + NT < NA) {
+                    xo_next = ld_relaxed_b32(X + v + NT);
+                    if constexpr (!BF) dg_next = ld_stream_f32(p.degf + v + NT);
+                }
+                const int e = r < NA ? rend[r] - b0 : 0, eb = r > 0 && r < NA ? rend[r - 1] - b0 : 0;
+                const uint32_t sum = row_sum<MODE>(sh, buf, E, e, eb, r == 0 ? row0 : Op<MODE>::identity());
+                if (r >= NA) continue;
                 if constexpr (FRONTIER) {
                     if (shared) {
-                        const uint32_t sum = sh.rowsum[r];
                         const uint32_t prev = atomicMin(X + v, sum);
                         if (sum < prev) {
                             res_part += 1.0f;
@@ -446,21 +465,12 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_tma_kernel(const SweepPar
                         continue;
                     }
                 }
-                uint32_t xo_bits;
-                float dg = 0.0f;
-                if (k == 0) {  // the first NT rows' inputs came with the tile
-                    xo_bits = old[r];
-                    if constexpr (!BF) dg = __uint_as_float(degs[r]);
-                } else {
-                    xo_bits = ld_relaxed_b32(X + v);
-                    if constexpr (!BF) dg = ld_stream_f32(p.degf + v);
-                }
-                const uint32_t xnew = row_update<MODE>(p, v, sh.rowsum[r], xo_bits, dg, gt, A.off_f, res_part, g_part,
-                                                       dg_part);
+                const uint32_t xnew = row_update<MODE>(p, v, sum, xo_bits, dg, gt, A.off_f, res_part, g_part, dg_part);
                 if constexpr (FRONTIER)  // the row goes on the CTA's list; its marks are counted at the sweep's end
                     log_changed(p.fr_chg + row_lo, &sh.nchg, xnew < xo_bits, v, epilogue_lanes(NA, k));
                 st_relaxed_b32(X + v, xnew);
             }
+            buf ^= 1;
             if constexpr (LIVE_G) {  // this tile's change of N: one share per warp, added after barrier (A)
                 const float s = warp_sum(dg_part);
                 dg_part = 0.0f;
@@ -468,15 +478,12 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_tma_kernel(const SweepPar
             }
         }  // tiles
         qbase += ntl;
-        if constexpr (LIVE_G) {
-            __syncthreads();  // the last tile's shares
-            flush_dg(sh, sb, c, L.S);
-        }
+        __syncthreads();  // the last tile's rows are done with val (block_add), its shares of N are there
+        if constexpr (LIVE_G) flush_dg(sh, sb, c, L.S);
 
         // -------- end of sweep: residual, barrier, stopping rule (frontier: tile marks) --------
         if constexpr (FRONTIER) {
             if (!shared) {  // an own sweep's changed rows are on the CTA's list (a shared sweep counted them)
-                __syncthreads();
                 marks += changed_marks(p.fr_chg + row_lo, sh.nchg, p.fr_orow);
             }
         }
