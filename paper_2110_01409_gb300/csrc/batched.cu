@@ -475,7 +475,7 @@ void release_batched_graphs(const dag_plan* plan)
 // columns (RMAT, 1 M vertices) 27.4, 27.1, 28-30, 29.7, 34.6 ms; of 64 columns (uniform, 262 K) 6.0, 4.9, 4.3, 4.1,
 // 3.9 ms; of 20 columns (RMAT, 100 K) 2.0, 1.4, 1.3, 1.3, 1.3 ms; Bellman-Ford of 64 columns (RMAT, 1 M) 7.1, 6.9,
 // 7.1, 7.1, 7.1 ms.
-constexpr int RUN_MIN_ITEMS = 64;
+constexpr int RUN_MIN_ITEMS = 16;
 constexpr int RUN_ITEMS = 1024;
 constexpr int RUN_ITEMS_WIDE = 256;
 

@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(NT, run_min_blocks(LPR, CH)) batched_runs_kern
                 ok = __all_sync(FULL, got) != 0;
                 if (!ok) break;
                 const unsigned have = __ballot_sync(FULL, full);
-                __threadfence();  // the flags before the partials
+                fence_gpu();  // the flags before the partials
                 for (int l = grp; l < n_back; l += GRP) {
                     if (!((have >> l) & 1u)) continue;
 #pragma unroll
@@ -716,7 +716,7 @@ __global__ void __launch_bounds__(NT, run_min_blocks(LPR, CH)) batched_runs_kern
             for (int q = 0; q < CH; ++q)
                 if (has(q)) st_relaxed_v4(p.part + (size_t)t * S + col0(q), acc[q]);
         }
-        if (some) __threadfence();
+        if (some) fence_gpu();
         __syncwarp();
         if (lane == 0) st_pub(p.pub + t, ((unsigned long long)stamp << 32) | (some ? 0u : PUB_EMPTY));
         // the pending row is finished a run later, by when the runs before it have published theirs (a run publishes

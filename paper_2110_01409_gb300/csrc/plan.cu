@@ -389,7 +389,9 @@ int get_warp_partition_range(dag_plan* plan, int W, int tile, int row_w, int lo,
 
 // Runs of the batched kernels: run w of W starts at w / W of the merge path's
 // weight, a row's end weighing row_w and an in-edge 1 (a cut inside a row's end
-// goes before it). Rows [run_row[w], run_row[w + 1]) end in run w.
+// goes before it), or, inside a row of at most a quarter of a run, at the row's
+// nearer end: only longer rows are split over runs, whose partials have to be
+// published and looked back for. Rows [run_row[w], run_row[w + 1]) end in run w.
 __global__ void k_batch_runs(const int* rowptr, int n, long long total, int row_w, int W, int* run_row, int* run_nz)
 {
     const int w = blockIdx.x * blockDim.x + threadIdx.x;
@@ -401,8 +403,17 @@ __global__ void k_batch_runs(const int* rowptr, int n, long long total, int row_
         if ((long long)row_w * (mid + 1) + rowptr[mid + 1] > target) hi = mid;
         else lo = mid + 1;
     }
+    int nz = rowptr[n];
+    if (lo < n) {
+        const int r0 = rowptr[lo], r1 = rowptr[lo + 1];
+        nz = (int)min(target - (long long)row_w * lo, (long long)r1);
+        if (4LL * (r1 - r0) <= total / W) {
+            if (2 * (nz - r0) > r1 - r0) { nz = r1; ++lo; }
+            else nz = r0;
+        }
+    }
     run_row[w] = lo;
-    run_nz[w] = lo == n ? rowptr[n] : (int)min(target - (long long)row_w * lo, (long long)rowptr[lo + 1]);
+    run_nz[w] = nz;
 }
 
 int get_batch_runs(dag_plan* plan, int W, int row_w, Partition** out, cudaStream_t s)
