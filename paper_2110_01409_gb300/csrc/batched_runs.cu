@@ -19,8 +19,9 @@
 // columns) and were 5 to 30% slower.
 //
 // Measured (RMAT, against a CTA block of whole rows walked in tiles by eight warps with a barrier per tile, and a
-// warp of 32 columns for other column counts): PPR of 256 columns at 1 M vertices 66.5 -> 27.1 ms, of 20 columns at
-// 100 K vertices 7.06 -> 1.33 ms (a hub's row was one warp's), Bellman-Ford of 64 columns at 1 M vertices 24.4 -> 7.1.
+// warp of 32 columns for other column counts): PPR of 256 columns at 1 M vertices 66.5 -> 27.3 ms, of 20 columns at
+// 100 K vertices 7.06 -> 1.19 ms (a hub's row was one warp's), Bellman-Ford of 64 columns at 1 M vertices 24.4 -> 7.5.
+// Slower than that kernel on small uniform graphs of 32 columns only (3 K vertices, PPR: 165 -> 200 us).
 //
 // Bellman-Ford reads only what can lower something: chg[u] is the last sweep that lowered any of u's columns, and
 // a sweep skips an in-edge whose source changed neither in it nor in the one before (its value is already in the
@@ -112,14 +113,17 @@ __device__ __forceinline__ unsigned below(int k) { return k >= 32 ? 0xffffffffu 
 
 }  // namespace
 
-constexpr int run_min_blocks(int LPR, int CH) { return CH >= 4 ? 1 : CH == 2 ? 2 : 3; }
-// Ring slots per warp: two batches, 8 KB of rows at most (16 KB above 512 columns).
-constexpr int run_depth(int LPR, int CH) { return CH >= 4 ? 4 : CH == 2 ? 8 : LPR == 32 ? 16 : 32; }
+constexpr int run_min_blocks(bool BF, int CH) { return CH >= 4 ? 1 : CH == 2 || !BF ? 2 : 3; }
+// CTAs per SM the registers are sized for: PPR at two (three spilled up to 64 bytes: 64 columns, uniform, 20 K vertices
+// 483 -> 346 us; RMAT, 400 K, 7.1 -> 4.3 ms), Bellman-Ford, which waits for last-change bytes, at three.
+// Ring slots per warp: two batches, 4 to 8 KB of rows (16 KB above 512 columns). 8 KB for 64 columns left three CTAs
+// 28 KB of L1: Bellman-Ford uniform 20 K 615 -> 490 us with half of it (RMAT 1 M 7.1 -> 7.5 ms).
+constexpr int run_depth(int LPR, int CH) { return CH >= 4 ? 4 : CH == 2 ? 8 : LPR >= 16 ? 16 : 32; }
 
 // LPR lanes hold a row (four columns per lane and chunk), CH chunks per lane (more than one only with LPR = 32);
 // WHOLE: the row fills them all, so its length is a constant.
 template <bool BF, int LPR, int CH, bool WHOLE>
-__global__ void __launch_bounds__(NT, run_min_blocks(LPR, CH)) batched_runs_kernel(const BatchParams p)
+__global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kernel(const BatchParams p)
 {
     constexpr unsigned FULL = 0xffffffffu;
     constexpr int GRP = 32 / LPR;          // in-edges a warp adds at a time
@@ -254,6 +258,9 @@ __global__ void __launch_bounds__(NT, run_min_blocks(LPR, CH)) batched_runs_kern
     }
     __syncthreads();
 
+    // the warp's first run is the same in every sweep
+    const int first_i0 = p.run_row[w], first_ie = p.run_row[w + 1], first_j0 = p.run_nz[w], first_je = p.run_nz[w + 1];
+    const bool first_head = first_j0 > p.rowptr[first_i0] && first_ie > first_i0;
     int it = 0;
     for (; it < p.max_iters; ++it) {
         const int slot = it % 3;
@@ -434,15 +441,15 @@ __global__ void __launch_bounds__(NT, run_min_blocks(LPR, CH)) batched_runs_kern
             return ok;
         };
 
-        if (!BF && !sync) live(true);
         int stages = 0;
         int pend = -1, pend_row = 0;  // the run whose first row waits for earlier runs' partials
         bool ok = true;
         for (int t = w; t < p.nruns && ok; t += W) {
         // ---------------- run t, as a stream of fetches ----------------
-        const int i0 = p.run_row[t], i_end = p.run_row[t + 1];  // rows [i0, i_end) end in this run
-        const int j0 = p.run_nz[t], j_end = p.run_nz[t + 1];
-        const bool head = j0 > p.rowptr[i0] && i_end > i0;      // it starts inside row i0 and ends it
+        // rows [i0, i_end) end in this run; head: it starts inside row i0 and ends it
+        const int i0 = t == w ? first_i0 : p.run_row[t], i_end = t == w ? first_ie : p.run_row[t + 1];
+        const int j0 = t == w ? first_j0 : p.run_nz[t], j_end = t == w ? first_je : p.run_nz[t + 1];
+        const bool head = t == w ? first_head : j0 > p.rowptr[i0] && i_end > i0;
         int i = i0, j = j0, ph = 0;   // next row end, next in-edge, 1: row i's old values are behind, its V ahead
         bool carry_need = false;      // BF: the row in progress has a kept in-edge in an earlier stage
         bool head_pending = head;
@@ -461,6 +468,7 @@ __global__ void __launch_bounds__(NT, run_min_blocks(LPR, CH)) batched_runs_kern
             }
         };
         load_raw();
+        if (!BF && !sync && t == w) live(true);  // (while the first loads of the sweep are in flight)
         // The next items of the run into list half lb (all of them, or for Bellman-Ford the ones a sweep needs);
         // an empty stage means that the run is done.
         auto build = [&](int lb) -> RunStage {
