@@ -26,31 +26,29 @@ int cuda_check(cudaError_t e, const char* what)
 
 namespace {
 
+// Device time of a solve, by the plan's two events (made once, destroyed with the plan).
 struct Timer {
-    cudaEvent_t a = nullptr, b = nullptr;
-    bool on = false;
-    void start(cudaStream_t s, bool want)
+    cudaEvent_t* ev = nullptr;
+    void start(dag_plan* plan, cudaStream_t s, bool want)
     {
-        on = want;
-        if (!on) return;
-        cudaEventCreate(&a);
-        cudaEventCreate(&b);
-        cudaEventRecord(a, s);
+        if (!want) return;
+        for (cudaEvent_t& e : plan->ev)
+            if (!e && cudaEventCreate(&e) != cudaSuccess) {
+                cudaGetLastError();
+                return;
+            }
+        ev = plan->ev;
+        cudaEventRecord(ev[0], s);
     }
     void stop(cudaStream_t s)
     {
-        if (on) cudaEventRecord(b, s);
+        if (ev) cudaEventRecord(ev[1], s);
     }
     float ms()
     {
         float x = 0.0f;
-        if (on) cudaEventElapsedTime(&x, a, b);
+        if (ev) cudaEventElapsedTime(&x, ev[0], ev[1]);
         return x;
-    }
-    ~Timer()
-    {
-        if (a) cudaEventDestroy(a);
-        if (b) cudaEventDestroy(b);
     }
 };
 
@@ -58,7 +56,7 @@ struct Timer {
 int finish_solve(dag_plan* plan, int nblocks, int delta, Timer& tm, cudaStream_t s, dag_stats* h, bool frontier = false)
 {
     SyncBlock sb;
-    DAG_CUDA(cudaMemcpyAsync(&sb, plan->sync, sizeof(SyncBlock), cudaMemcpyDeviceToHost, s));
+    DAG_CUDA(cudaMemcpyAsync(&sb, plan->sync, SYNC_HEAD, cudaMemcpyDeviceToHost, s));
     DAG_CUDA(cudaStreamSynchronize(s));
     DAG_CUDA(cudaGetLastError());
     int rc = DAG_OK;
@@ -164,7 +162,7 @@ extern "C" int dag_pagerank(dag_plan* plan, float d, double tol, dag_variant var
     p.warp = (flags & (DAG_WARP_WORKERS | DAG_WARP_ORDERED)) ? 1 : 0;
     p.ordered = (flags & DAG_WARP_ORDERED) ? 1 : 0;
     Timer tm;
-    tm.start(s, h_stats != nullptr);
+    tm.start(plan, s, h_stats != nullptr);
     int nb = 0;
     rc = launch_sweep(plan, d_val ? MODE_PRW : MODE_PR, var, delta, p, s, &nb);
     if (rc) return rc;
@@ -219,7 +217,7 @@ int sssp_impl(dag_plan* plan, uint32_t src, int variant, int delta, int max_iter
         if (rc) return rc;
     }
     Timer tm;
-    tm.start(s, h_stats != nullptr);
+    tm.start(plan, s, h_stats != nullptr);
     int nb = 0;
     rc = launch_sweep(plan, w8 ? MODE_BF8 : MODE_BF, var, delta, p, s, &nb);
     if (rc) return rc;
@@ -311,7 +309,7 @@ extern "C" int dag_pagerank_adjoint(dag_plan* in_plan, dag_plan* out_plan, float
     p.warp = (flags & (DAG_WARP_WORKERS | DAG_WARP_ORDERED)) ? 1 : 0;
     p.ordered = (flags & DAG_WARP_ORDERED) ? 1 : 0;
     Timer tm;
-    tm.start(s, true);
+    tm.start(out_plan, s, true);
     int nb = 0;
     rc = launch_sweep(out_plan, MODE_ADJ, var, delta, p, s, &nb);
     if (rc) {

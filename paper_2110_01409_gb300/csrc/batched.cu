@@ -504,20 +504,32 @@ int launch_batched(dag_plan* plan, int is_bf, int variant, int delta, int max_it
         threads_launch = NT;
         dyn = run_smem_bytes(is_bf != 0, B);
     }
-    int max_dyn = 0;
-    DAG_CUDA(cudaDeviceGetAttribute(&max_dyn, cudaDevAttrMaxSharedMemoryPerBlockOptin, plan->device));
-    if (dyn > (size_t)max_dyn)
-        return set_error(DAG_ERR_INVALID, "delta too large for the batched delay buffers in shared memory");
-    DAG_CUDA(cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
     int per_sm = 0;
-    DAG_CUDA(cudaFuncSetAttribute((const void*)k, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-    DAG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)k, threads_launch, dyn));
-    if (per_sm < 1) return set_error(DAG_ERR_INVALID, "batched kernel cannot be resident");
-    {
+    const auto fit = plan->batched_fit.find({(const void*)k, dyn});
+    if (fit != plan->batched_fit.end()) {
+        per_sm = fit->second.first;
+        Shape how;
+        how.kernels[0] = (const void*)k;
+        how.dyn = (int)dyn;
+        how.carveout = fit->second.second;
+        const int rc = apply_shape(how);
+        if (rc) return rc;
+    } else {
+        int max_dyn = 0;
+        DAG_CUDA(cudaDeviceGetAttribute(&max_dyn, cudaDevAttrMaxSharedMemoryPerBlockOptin, plan->device));
+        if (dyn > (size_t)max_dyn)
+            return set_error(DAG_ERR_INVALID, "delta too large for the batched delay buffers in shared memory");
+        DAG_CUDA(cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+        DAG_CUDA(cudaFuncSetAttribute((const void*)k, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+        DAG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)k, threads_launch, dyn));
+        if (per_sm < 1) return set_error(DAG_ERR_INVALID, "batched kernel cannot be resident");
         cudaFuncAttributes fa;
         DAG_CUDA(cudaFuncGetAttributes(&fa, (const void*)k));
-        const int rc = set_l1_carveout((const void*)k, plan->device, threads_launch, fa.sharedSizeBytes, dyn, per_sm);
+        int pct = 0;
+        const int rc =
+            set_l1_carveout((const void*)k, plan->device, threads_launch, fa.sharedSizeBytes, dyn, per_sm, &pct);
         if (rc) return rc;
+        plan->batched_fit[{(const void*)k, dyn}] = {per_sm, pct};
     }
     int nb = per_sm * plan->num_sms;
     if (plan->worker_cap > 0 && nb > plan->worker_cap) nb = plan->worker_cap;
@@ -623,32 +635,25 @@ int launch_batched(dag_plan* plan, int is_bf, int variant, int delta, int max_it
         p.part = (uint32_t*)plan->bruns;
         p.chg = (uint8_t*)plan->bruns + part_bytes;
     }
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (st) {
-        cudaEventCreate(&e0);
-        cudaEventCreate(&e1);
-        cudaEventRecord(e0, s);
+        for (cudaEvent_t& e : plan->ev)
+            if (!e) DAG_CUDA(cudaEventCreate(&e));
+        cudaEventRecord(plan->ev[0], s);
     }
     void* args[] = {(void*)&p};
     bool replayed = false;
     cudaError_t le = use_graph ? graph_launch(plan, (const void*)k, nb, threads_launch, dyn, cbytes, args, s, &replayed)
                                : cudaLaunchCooperativeKernel((const void*)k, dim3(nb), dim3(threads_launch), args, dyn, s);
-    if (le != cudaSuccess) {
-        if (e0) cudaEventDestroy(e0);
-        if (e1) cudaEventDestroy(e1);
-        return cuda_check(le, "batched cooperative launch");
-    }
+    if (le != cudaSuccess) return cuda_check(le, "batched cooperative launch");
     if (!st) return DAG_OK;
-    cudaEventRecord(e1, s);
+    cudaEventRecord(plan->ev[1], s);
     SyncBlock sb;
-    DAG_CUDA(cudaMemcpyAsync(&sb, plan->bsync, sizeof(SyncBlock), cudaMemcpyDeviceToHost, s));
+    DAG_CUDA(cudaMemcpyAsync(&sb, plan->bsync, SYNC_HEAD, cudaMemcpyDeviceToHost, s));
     std::vector<int> hit(B);
     DAG_CUDA(cudaMemcpyAsync(hit.data(), iters, (size_t)B * sizeof(int), cudaMemcpyDeviceToHost, s));
     DAG_CUDA(cudaStreamSynchronize(s));
     float ms = 0.0f;
-    cudaEventElapsedTime(&ms, e0, e1);
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
+    cudaEventElapsedTime(&ms, plan->ev[0], plan->ev[1]);
     int rc2 = DAG_OK;
     if (sb.err) rc2 = sb.err;
     else if (!sb.converged) rc2 = DAG_ERR_NOT_CONVERGED;

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include <functional>
@@ -71,6 +72,9 @@ struct __align__(128) SyncBlock {
     int pad2[3];
     alignas(128) long long stripe[GSTRIPES * GSTRIDE];  // live global sum, fixed point (async / delayed)
 };
+
+// The bytes in front of the stripes: all that a host reads of a finished solve.
+constexpr size_t SYNC_HEAD = offsetof(SyncBlock, stripe);
 
 // Parameters of one sweep launch.
 struct SweepParams {
@@ -155,6 +159,17 @@ struct Partition {
     unsigned long long* tpub = nullptr;  // ordered warp sweeps: [tiles] published partials (built on first use)
 };
 
+// A settled launch shape, cached per plan: grid, delay buffer, partition, and how its kernels are configured. The
+// configuration is a kernel's, not a plan's, and another shape may have changed it since: it is set again before each
+// launch, without the queries that led to it.
+struct Shape {
+    int nb = 0, cap = 0, clamped = 0;
+    Partition* part = nullptr;
+    const void* kernels[2] = {nullptr, nullptr};
+    int dyn = 0;       // dynamic shared memory, bytes
+    int carveout = 0;  // shared-memory share of the SM's array, per cent
+};
+
 }  // namespace dag
 
 struct dag_plan {
@@ -186,6 +201,9 @@ struct dag_plan {
     int nw_nhubs = 0;
     void* grad_coef = nullptr;  // [n] float2 (d r_u / s_u, (M^T lambda)_u) of the edge gradients, first use
     std::map<long long, dag::Partition> parts;  // key: nblocks | row_cap << 32
+    std::map<std::tuple<int, int, int, int, int, int>, dag::Shape> shapes;  // see sweep_shape, warp_shape
+    std::map<std::pair<const void*, size_t>, std::pair<int, int>> batched_fit;  // (kernel, dyn) -> CTAs per SM, carveout
+    cudaEvent_t ev[2] = {nullptr, nullptr};  // around a solve whose time is asked for
     std::map<std::tuple<int, int, int, int>, dag::Partition> range_parts;  // (warps, tile, lo, hi)
     // batched workspace (grown on demand)
     void* bx = nullptr;
@@ -212,7 +230,7 @@ int get_partition(dag_plan* plan, int nblocks, Partition** out, cudaStream_t s, 
 
 // The frontier maps of a partition (and the plan's out-CSR row pointers), built once.
 int frontier_maps(dag_plan* plan, Partition* part, cudaStream_t s, bool with_end = true);
-int max_workers(dag_plan* plan, int mode, int variant, int buf_cap_elems, int* out);
+int max_workers(dag_plan* plan, int mode, int variant, int buf_cap_elems, int* out, Shape* how = nullptr);
 
 // sweep.cu
 int launch_sweep(dag_plan* plan, int mode, int variant, int delta, SweepParams& p, cudaStream_t s,
@@ -223,7 +241,7 @@ int sweep_shape(dag_plan* plan, int mode, int variant, int delta, int* nb_out, i
 // (`partition(nblocks, &max_rows)`), for launches without a plan's workspace.
 int settle_shape(dag_plan* plan, int mode, int variant, int delta,
                  const std::function<int(int nblocks, int* max_rows)>& partition, int* nb_out, int* cap_out,
-                 int* clamped_out);
+                 int* clamped_out, Shape* how = nullptr);
 // Rows a tile of a delayed sweep may complete (0: no cap): a buffer of delta
 // rows can only be flushed at a tile end.
 inline int delayed_row_cap(int variant, int delta) { return (variant == DAG_DELAYED && delta > 0 && delta < TILE) ? delta : 0; }
@@ -238,7 +256,10 @@ const void* sweep_tma_kernel_ptr(int mode, bool frontier);
 size_t sweep_tma_ring_bytes(int mode);
 // Smallest shared-memory carveout of kernel k that keeps per_sm CTAs of
 // (static_smem + dyn) bytes resident; the rest of the SM's array is L1.
-int set_l1_carveout(const void* k, int device, int threads, size_t static_smem, size_t dyn, int per_sm);
+int set_l1_carveout(const void* k, int device, int threads, size_t static_smem, size_t dyn, int per_sm,
+                    int* pct_out = nullptr);
+// Configures a cached shape's kernels as they were when it settled.
+int apply_shape(const Shape& sh);
 
 // Warp workers: the whole merge path cut into tiles of `tile` items, warp w
 // of W taking the run of tiles from w / W to (w + 1) / W of the path's weight

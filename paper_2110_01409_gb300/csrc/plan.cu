@@ -792,6 +792,8 @@ extern "C" int dag_plan_destroy(dag_plan* p)
     cudaFree(p->bx);  // batched workspace: cudaMalloc (batched.cu)
     cudaFree(p->bsync);
     dev_free(p->bruns);
+    for (cudaEvent_t e : p->ev)
+        if (e) cudaEventDestroy(e);
     for (auto& kv : p->parts) {
         dev_free(kv.second.cta_row);
         dev_free(kv.second.cta_tile);

@@ -465,7 +465,7 @@ size_t sweep_ring_bytes(int mode, int variant) { return variant == DAG_ASYNC ? s
 // Without a preference the driver may keep whatever L1/shared split an earlier
 // kernel needed (up to the largest shared share), which leaves L1 small and
 // makes a sweep's speed depend on what ran before it.
-int set_l1_carveout(const void* k, int device, int threads, size_t static_smem, size_t dyn, int per_sm)
+int set_l1_carveout(const void* k, int device, int threads, size_t static_smem, size_t dyn, int per_sm, int* pct_out)
 {
     int max_sm = 0, reserved = 0;
     DAG_CUDA(cudaDeviceGetAttribute(&max_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, device));
@@ -476,14 +476,28 @@ int set_l1_carveout(const void* k, int device, int threads, size_t static_smem, 
     DAG_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, pct));
     int got = 0;
     DAG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&got, k, threads, dyn));
-    if (got < per_sm) DAG_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+    if (got < per_sm) {
+        pct = 100;
+        DAG_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, pct));
+    }
+    if (pct_out) *pct_out = pct;
+    return DAG_OK;
+}
+
+int apply_shape(const Shape& sh)
+{
+    for (const void* k : sh.kernels) {
+        if (!k) continue;
+        DAG_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sh.dyn));
+        DAG_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, sh.carveout));
+    }
     return DAG_OK;
 }
 
 // CTAs of a (mode, variant) sweep that fit on the GPU at once, with each kernel
 // such a solve may run (plain, and frontier for Bellman-Ford) configured for
 // that residency: dynamic shared memory and L1/shared carveout.
-int max_workers(dag_plan* plan, int mode, int variant, int buf_cap_elems, int* out)
+int max_workers(dag_plan* plan, int mode, int variant, int buf_cap_elems, int* out, Shape* how)
 {
     const void* ks[2] = {(const void*)kernel_for(mode, variant, false), (const void*)kernel_for(mode, variant, true)};
     const int nk = ks[1] != ks[0] ? 2 : 1;
@@ -519,8 +533,14 @@ int max_workers(dag_plan* plan, int mode, int variant, int buf_cap_elems, int* o
         while (per_sm > 1 && (size_t)per_sm * per_cta > budget) --per_sm;
     }
     for (int i = 0; i < nk; ++i) {
-        const int rc = set_l1_carveout(ks[i], plan->device, NT, fa.sharedSizeBytes, dyn, per_sm);
+        int pct = 0;
+        const int rc = set_l1_carveout(ks[i], plan->device, NT, fa.sharedSizeBytes, dyn, per_sm, &pct);
         if (rc) return rc;
+        if (how) {
+            how->kernels[i] = ks[i];
+            how->dyn = (int)dyn;
+            how->carveout = std::max(i == 0 ? 0 : how->carveout, pct);
+        }
     }
     *out = per_sm * plan->num_sms;
     return DAG_OK;
@@ -536,10 +556,10 @@ int max_workers(dag_plan* plan, int mode, int variant, int buf_cap_elems, int* o
 // largest block's row count.
 int settle_shape(dag_plan* plan, int mode, int variant, int delta,
                  const std::function<int(int nblocks, int* max_rows)>& partition, int* nb_out, int* cap_out,
-                 int* clamped_out)
+                 int* clamped_out, Shape* how)
 {
     int nb = 0;
-    int rc = max_workers(plan, mode, variant, 0, &nb);
+    int rc = max_workers(plan, mode, variant, 0, &nb, how);
     if (rc) return rc;
     {
         // A small graph's sweep is its grid barrier: one CTA per tile (two at least, so that a barrier has someone to
@@ -572,7 +592,7 @@ int settle_shape(dag_plan* plan, int mode, int variant, int delta,
         clamped = need < want ? 1 : 0;
         cap = (int)(need < 1 ? 1 : need);
         int nb2 = 0;
-        rc = max_workers(plan, mode, variant, cap, &nb2);
+        rc = max_workers(plan, mode, variant, cap, &nb2, how);
         if (rc) return rc;
         if (nb2 < nb) {
             nb = nb2;
@@ -591,6 +611,17 @@ int settle_shape(dag_plan* plan, int mode, int variant, int delta,
 int sweep_shape(dag_plan* plan, int mode, int variant, int delta, int* nb_out, int* cap_out, Partition** part_out,
                 cudaStream_t s, int* clamped_out)
 {
+    const auto key = std::make_tuple(0, mode, variant, variant == DAG_DELAYED ? delta : 0, plan->worker_cap, 0);
+    const auto it = plan->shapes.find(key);
+    if (it != plan->shapes.end()) {
+        const Shape& sh = it->second;
+        *nb_out = sh.nb;
+        *cap_out = sh.cap;
+        *part_out = sh.part;
+        if (clamped_out) *clamped_out = sh.clamped;
+        return apply_shape(sh);
+    }
+    Shape sh;
     Partition* part = nullptr;
     int clamped = 0;
     auto build = [&](int nb, int* max_rows) {
@@ -598,9 +629,14 @@ int sweep_shape(dag_plan* plan, int mode, int variant, int delta, int* nb_out, i
         if (rc == DAG_OK) *max_rows = part->max_rows;
         return rc;
     };
-    const int rc = settle_shape(plan, mode, variant, delta, build, nb_out, cap_out, &clamped);
+    const int rc = settle_shape(plan, mode, variant, delta, build, nb_out, cap_out, &clamped, &sh);
     if (rc) return rc;
     *part_out = part;
+    sh.nb = *nb_out;
+    sh.cap = *cap_out;
+    sh.clamped = clamped;
+    sh.part = part;
+    plan->shapes.emplace(key, sh);
     if (clamped_out) *clamped_out = clamped;
     return DAG_OK;
 }

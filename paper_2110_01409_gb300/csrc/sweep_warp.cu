@@ -625,6 +625,18 @@ static int warp_shape(dag_plan* plan, int mode, int variant, int delta, int* nb_
     const int WTILE = 32 * plan->warp_ipt;
     const void* k = warp_kernel(kind, mode, variant, plan->warp_ipt, ordered);
     if (!k) return set_error(DAG_ERR_INVALID, "no warp tile of that shape");
+    const auto key = std::make_tuple(1 + kind + (ordered ? 8 : 0), mode, variant, variant == DAG_DELAYED ? delta : 0,
+                                     plan->worker_cap, plan->warp_ipt);
+    const auto hit = plan->shapes.find(key);
+    if (hit != plan->shapes.end()) {
+        const Shape& sh = hit->second;
+        *nb_out = sh.nb;
+        *cap_out = sh.cap;
+        *clamped_out = sh.clamped;
+        *part_out = sh.part;
+        return apply_shape(sh);
+    }
+    Shape sh;
     cudaFuncAttributes fa{};
     DAG_CUDA(cudaFuncGetAttributes(&fa, k));
     int max_dyn = 0;
@@ -639,8 +651,9 @@ static int warp_shape(dag_plan* plan, int mode, int variant, int delta, int* nb_
         int per_sm = 0;
         DAG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, NT, dyn));
         if (per_sm < 1) return set_error(DAG_ERR_INVALID, "warp sweep cannot be resident with this delta");
-        const int rc = set_l1_carveout(k, plan->device, NT, fa.sharedSizeBytes, dyn, per_sm);
+        const int rc = set_l1_carveout(k, plan->device, NT, fa.sharedSizeBytes, dyn, per_sm, &sh.carveout);
         if (rc) return rc;
+        sh.dyn = (int)dyn;
         int n_cta = per_sm * plan->num_sms;
         // a small graph's sweep is its grid barrier: one tile per warp (two CTAs at least), as settle_shape; 5,000
         // vertices in 608 CTAs took 545 us, the runs' look-back waiting along runs without a tile, in 34 112
@@ -676,6 +689,12 @@ static int warp_shape(dag_plan* plan, int mode, int variant, int delta, int* nb_
     *cap_out = cap;
     *clamped_out = clamped;
     *part_out = part;
+    sh.nb = nb;
+    sh.cap = cap;
+    sh.clamped = clamped;
+    sh.part = part;
+    sh.kernels[0] = k;
+    plan->shapes.emplace(key, sh);
     return DAG_OK;
 }
 
