@@ -5,8 +5,11 @@
 // A pass over the vertices packs each source's two factors, d r_u / s_u and
 // (M^T lambda)_u, into one 8-byte pair; then one pass over the in-edges in the
 // caller's (in-CSR) order, one gather per edge: each CTA walks its vertex
-// block tile by tile and finds an edge's row by binary search over the tile's
-// row ends in shared memory.
+// block tile by tile. An edge's row is the last one starting at or before it:
+// rows leave their number at their first edge, and a running maximum over the
+// warp's edges spreads it (a binary search over the tile's row ends per edge
+// took 250 us for 33.5 M edges, this takes 216; one gather per SM clock would be
+// 110).
 #include <climits>
 
 #include "dag_internal.cuh"
@@ -24,26 +27,48 @@ __global__ void __launch_bounds__(NT) k_edge_grad(const int* rowptr, const int* 
                                                   const int* tile_row, const int* tile_nz, const float2* coef,
                                                   const float* lambda, float* grad_w)
 {
-    __shared__ int s_end[TILE + 1];
-    const int c = blockIdx.x;
+    __shared__ int s_row[TILE];       // 1 + the row (from a0) whose first edge in the tile this is, else 0
+    __shared__ int s_last[NWARP];     // the last row started in each warp's part of the tile
+    constexpr int PART = TILE / NWARP;  // edges per warp, IPT per lane, 32 at a time
+    const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int t = cta_tile[c]; t < cta_tile[c + 1]; ++t) {
         const int a0 = tile_row[t], b0 = tile_nz[t];
         const int NA = tile_row[t + 1] - a0, NB = tile_nz[t + 1] - b0;
+        int col[IPT];
+#pragma unroll
+        for (int q = 0; q < IPT; ++q) {
+            const int j = warp * PART + 32 * q + lane;
+            col[q] = j < NB ? colidx[b0 + j] : -1;
+        }
+        __syncthreads();  // the previous tile's rows are read
+        for (int j = tid; j < NB; j += NT) s_row[j] = 0;
         __syncthreads();
-        for (int i = threadIdx.x; i < NA; i += NT) s_end[i] = rowptr[a0 + i + 1] - b0;
-        if (threadIdx.x == 0) s_end[NA] = INT_MAX;  // the row still open at the tile's end
+        // row i starts where row i - 1 ends (the first at the tile's first edge); row NA goes on past the tile
+        for (int i = tid; i <= NA; i += NT) {
+            const int b = i > 0 ? rowptr[a0 + i] - b0 : 0, e = i < NA ? rowptr[a0 + i + 1] - b0 : NB;
+            if (b < e) s_row[b] = i + 1;
+        }
         __syncthreads();
-        for (int j = threadIdx.x; j < NB; j += NT) {
-            // row of edge j: first i with s_end[i] > j
-            int lo = 0, hi = NA;
-            while (lo < hi) {
-                int mid = (lo + hi) >> 1;
-                if (s_end[mid] > j) hi = mid;
-                else lo = mid + 1;
-            }
-            const int e = b0 + j;
-            const float2 cf = coef[colidx[e]];
-            grad_w[e] = cf.x * (lambda[a0 + lo] - cf.y);
+        int m[IPT], run = 0;
+#pragma unroll
+        for (int q = 0; q < IPT; ++q) {
+            const int j = warp * PART + 32 * q + lane;
+            int v = j < NB ? s_row[j] : 0;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) v = max(v, __shfl_up_sync(0xffffffffu, v, o));  // (below lane o: its own)
+            m[q] = max(v, run);
+            run = __shfl_sync(0xffffffffu, m[q], 31);
+        }
+        if (lane == 0) s_last[warp] = run;
+        __syncthreads();
+        int before = 0;
+        for (int k = 0; k < warp; ++k) before = max(before, s_last[k]);
+#pragma unroll
+        for (int q = 0; q < IPT; ++q) {
+            const int j = warp * PART + 32 * q + lane;
+            if (col[q] < 0) continue;
+            const float2 cf = coef[col[q]];
+            grad_w[b0 + j] = cf.x * (lambda[a0 + max(m[q], before) - 1] - cf.y);
         }
     }
 }

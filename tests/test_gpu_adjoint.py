@@ -196,3 +196,40 @@ def test_adjoint_deflation_cuts_the_slow_mode(dag, scaled_case, variant, delta, 
     assert st2["iters"] <= 2 * st["iters"]
     assert _rel(gw.cpu().numpy(), gw_ref) <= 1e-4
     assert _rel(gt.cpu().numpy(), gt_ref) <= 1e-4
+
+
+def test_normalisation_and_edge_gradients_at_the_kernels_edges(dag):
+    # sources of 0, 1, 8, 63 .. 65, 2047 .. 2049 and 5000 out-edges (eight lanes, a warp, a block per source); in-edge
+    # tiles inside one row, with runs of empty rows, and ending at a row's end
+    n = 6000
+    degs = {0: 1, 1: 8, 2: 63, 3: 64, 4: 65, 5: 2047, 6: 2048, 7: 2049, 8: 5000}
+    rng = np.random.default_rng(4)
+    src = np.concatenate([np.full(k, u) for u, k in degs.items()] + [np.arange(9, 5400)])
+    dst = np.concatenate([rng.permutation(np.arange(9, n))[:k] for k in degs.values()] + [np.full(5391, 5999)])
+    keep = src != dst
+    g = I.from_edges(n, src[keep], dst[keep])
+    plan = dag.Plan.from_graph(g, "cuda")
+    w = torch.rand(g.m, generator=torch.Generator().manual_seed(1)).add_(0.1).cuda()
+    val, s = dag.normalize_weights(plan, w)
+    col = plan.colidx.long()
+    ref = torch.zeros(n, dtype=torch.float64, device="cuda").index_add_(0, col, w.double())
+    # a source's FP32 sum of k terms: at most 160 additions in a row, 160 * 2^-24 < 1e-5
+    assert torch.allclose(s.double(), ref, rtol=1e-5, atol=0)
+    assert torch.allclose(val.double(), w.double() / ref[col], rtol=2e-5, atol=0)
+    val2, s2 = dag.normalize_weights(plan, w)
+    assert torch.equal(s, s2) and torch.equal(val, val2)
+    orow, ocol, perm = dag.transpose(plan)
+    out_plan = dag.Plan(orow, ocol)
+    r, _ = dag.pagerank(plan, 0.85, 1e-6, "sync", 0, val=val)
+    c = torch.rand(n, generator=torch.Generator().manual_seed(2)).cuda()
+    gw, gt, lam, _ = dag.pagerank_adjoint(plan, out_plan, val, val[perm.long()].contiguous(), s, r, c, 0.85, 1e-7, "sync",
+                                          0, want_lambda=True)
+    dst_of = torch.repeat_interleave(torch.arange(n, device="cuda"), (plan.rowptr[1:] - plan.rowptr[:-1]).long())
+    lam64, val64 = lam.double(), val.double()
+    mt = torch.zeros(n, dtype=torch.float64, device="cuda").index_add_(0, col, val64 * lam64[dst_of])
+    want = 0.85 * (r.double() / s.double())[col] * (lam64[dst_of] - mt[col])
+    # lambda and M^T lambda are FP32 values of size max|lambda|: their difference is good to a few of their roundings,
+    # and the sweep's M^T lambda is of the iterate before, 1e-7 of |c|_1 = n / 2 away at most
+    scale = float((r / s).nan_to_num(0, 0, 0)[col].abs().max()) * float(lam.abs().max())
+    assert float((gw.double() - want).abs().max()) <= 2e-4 * scale
+    assert torch.allclose(gt, 0.15 * lam, rtol=1e-6, atol=0)
