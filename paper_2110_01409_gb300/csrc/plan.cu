@@ -510,8 +510,11 @@ int launch_transpose(dag_plan* plan, int* out_rowptr, int* out_colidx, int* perm
 // [tile_nz[t], tile_nz[t+1]) of rows [tile_row[t], tile_row[t+1]]) takes the
 // next slot of u's out-list (cursor[u], one atomic per run of equal sources
 // in the warp) and writes there t and the tile ending row v: t itself for the
-// rows that end inside t, else the tile ending row tile_row[t+1] (oend may
-// be null).
+// rows that end inside t, else the tile ending row tile_row[t+1]. END false
+// leaves out the latter, and with it every edge's search for its row (RMAT 4 M
+// vertices: the first warp-tile frontier solve 3.47 -> 3.37 ms; the rest is an
+// atomic and a scattered store per edge).
+template <bool END>
 __global__ void k_frontier_scatter(const int* rowptr, const int* colidx, int n, const int* tile_row,
                                    const int* tile_nz, int tiles, int* cursor, int* otile, int* oend)
 {
@@ -523,7 +526,7 @@ __global__ void k_frontier_scatter(const int* rowptr, const int* colidx, int n, 
         if (nz0 >= nz1) continue;
         // the tile ending row r1: the first t' > t whose successor starts past r1
         int end1 = t;
-        if (r1 < n) {
+        if (END && r1 < n) {
             int lo = t + 1, hi = tiles - 1;
             while (lo < hi) {
                 const int mid = (lo + hi) >> 1;
@@ -538,7 +541,7 @@ __global__ void k_frontier_scatter(const int* rowptr, const int* colidx, int n, 
             const unsigned act = __ballot_sync(0xffffffffu, live);
             if (!live) continue;
             // the row of e: the last row of the tile starting at or before e
-            int lo = r0, hi = vmax;
+            int lo = r0, hi = END ? vmax : r0;
             while (lo < hi) {
                 const int mid = (lo + hi + 1) >> 1;
                 if (rowptr[mid] <= e) lo = mid; else hi = mid - 1;
@@ -551,7 +554,7 @@ __global__ void k_frontier_scatter(const int* rowptr, const int* colidx, int n, 
             base = __shfl_sync(peers, base, leader);
             const int pos = base + __popc(peers & ((1u << lane) - 1u));
             otile[pos] = t;
-            if (oend) oend[pos] = lo < r1 ? t : end1;
+            if (END) oend[pos] = lo < r1 ? t : end1;
         }
     }
 }
@@ -579,8 +582,9 @@ static int build_frontier_maps(dag_plan* plan, Partition* part, cudaStream_t s, 
         // fr_chg (a per-sweep list, written before it is read) serves as the cursor
         DAG_CUDA(cudaMemcpyAsync(part->fr_chg, plan->fr_orow, (size_t)n * sizeof(int), cudaMemcpyDeviceToDevice, s));
         const int blocks = (int)std::min(((long long)part->tiles * 32 + 255) / 256, 152LL * 64);
-        k_frontier_scatter<<<blocks, 256, 0, s>>>(plan->rowptr, plan->colidx, n, part->tile_row, part->tile_nz,
-                                                  part->tiles, part->fr_chg, part->fr_otile, part->fr_oend);
+        const auto scatter = with_end ? k_frontier_scatter<true> : k_frontier_scatter<false>;
+        scatter<<<blocks, 256, 0, s>>>(plan->rowptr, plan->colidx, n, part->tile_row, part->tile_nz, part->tiles,
+                                       part->fr_chg, part->fr_otile, part->fr_oend);
         DAG_CUDA(cudaGetLastError());
     }
     DAG_CUDA(cudaStreamSynchronize(s));
@@ -605,23 +609,53 @@ int frontier_maps(dag_plan* plan, Partition* part, cudaStream_t s, bool with_end
 }
 
 // s[u] = sum of w over u's out-edges, in a fixed order whatever the launch:
-// a warp per source (lane j takes out-edges j, j + 32, ... in out-CSR order,
-// then a butterfly of the lanes' sums); sources of more than NW_HUB out-edges
-// are left to k_out_sum_hub, a whole block per source.
+// eight lanes per source (lane j takes out-edges j, j + 8, ... in out-CSR
+// order, then a butterfly of the lanes' sums), sources of more than NW_WARP
+// out-edges by the whole warp in the same way, those of more than NW_HUB by
+// k_out_sum_hub, a whole block per source. Bound by the gathers w[perm[k]]; a
+// warp per source left most lanes idle (half of RMAT's sources have no
+// out-edge, most others fewer than 32): 345 -> 175 us for 2 M sources and 33.5 M
+// weights.
+constexpr int NW_WARP = 64;
 constexpr int NW_HUB = 2048;
 constexpr int NW_HUB_THREADS = 256;
 __global__ void k_out_sum(const int* orow, const int* perm, const float* w, int n, float* s)
 {
-    const int lane = threadIdx.x & 31;
-    const long long u = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-    if (u >= n) return;
-    const int k0 = orow[u], k1 = orow[u + 1];
-    if (k1 - k0 > NW_HUB) return;
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, sub = lane & 7;
+    const long long u = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 3;
+    const int k0 = u < n ? orow[u] : 0, k1 = u < n ? orow[u + 1] : 0, deg = k1 - k0;
     float acc = 0.0f;
-    for (int k = k0 + lane; k < k1; k += 32) acc += w[perm[k]];
+    if (deg <= NW_WARP) {
+        int k = k0 + sub;
+        for (; k + 24 < k1; k += 32) {  // four gathers in flight
+            const int p0 = perm[k], p1 = perm[k + 8], p2 = perm[k + 16], p3 = perm[k + 24];
+            const float a = w[p0], b = w[p1], c = w[p2], d = w[p3];
+            acc = acc + a + b + c + d;
+        }
+        for (; k < k1; k += 8) acc += w[perm[k]];
+    }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) s[u] = acc;
+    for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
+    if (sub == 0 && u < n && deg <= NW_WARP) s[u] = acc;
+    // the warp's longer sources, one after the other
+    unsigned longer = __ballot_sync(FULL, sub == 0 && deg > NW_WARP && deg <= NW_HUB);
+    while (longer) {
+        const int from = __ffs(longer) - 1;
+        longer &= longer - 1u;
+        const int b0 = __shfl_sync(FULL, k0, from), b1 = __shfl_sync(FULL, k1, from);
+        float t = 0.0f;
+        int k = b0 + lane;
+        for (; k + 96 < b1; k += 128) {
+            const int p0 = perm[k], p1 = perm[k + 32], p2 = perm[k + 64], p3 = perm[k + 96];
+            const float a = w[p0], b = w[p1], c = w[p2], d = w[p3];
+            t = t + a + b + c + d;
+        }
+        for (; k < b1; k += 32) t += w[perm[k]];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(FULL, t, o);
+        if (lane == from) s[u] = t;
+    }
 }
 __global__ void __launch_bounds__(NW_HUB_THREADS) k_out_sum_hub(const int* orow, const int* perm, const float* w,
                                                                const int* hubs, int nhubs, float* s)
@@ -632,7 +666,14 @@ __global__ void __launch_bounds__(NW_HUB_THREADS) k_out_sum_hub(const int* orow,
         const int u = hubs[h];
         const int k1 = orow[u + 1];
         float acc = 0.0f;
-        for (int k = orow[u] + threadIdx.x; k < k1; k += NW_HUB_THREADS) acc += w[perm[k]];
+        int k = orow[u] + threadIdx.x;
+        for (; k + 3 * NW_HUB_THREADS < k1; k += 4 * NW_HUB_THREADS) {  // four gathers in flight
+            const int p0 = perm[k], p1 = perm[k + NW_HUB_THREADS], p2 = perm[k + 2 * NW_HUB_THREADS],
+                      p3 = perm[k + 3 * NW_HUB_THREADS];
+            const float a = w[p0], b = w[p1], c = w[p2], d = w[p3];
+            acc = acc + a + b + c + d;
+        }
+        for (; k < k1; k += NW_HUB_THREADS) acc += w[perm[k]];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         if (lane == 0) part[wid] = acc;
@@ -701,7 +742,7 @@ int launch_normalize(dag_plan* plan, const float* w, float* val, float* s_out, c
         plan->nw_hubs = hubs;
         plan->nw_perm = perm;  // set last: a set nw_perm marks the out-CSR order complete
     }
-    k_out_sum<<<(unsigned)(((long long)n * 32 + 255) / 256), 256, 0, s>>>(plan->fr_orow, plan->nw_perm, w, n, s_out);
+    k_out_sum<<<(unsigned)(((long long)n * 8 + 255) / 256), 256, 0, s>>>(plan->fr_orow, plan->nw_perm, w, n, s_out);
     if (plan->nw_nhubs > 0)
         k_out_sum_hub<<<std::min(plan->nw_nhubs, 4 * plan->num_sms), NW_HUB_THREADS, 0, s>>>(
             plan->fr_orow, plan->nw_perm, w, plan->nw_hubs, plan->nw_nhubs, s_out);
