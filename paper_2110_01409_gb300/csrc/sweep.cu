@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_kernel(const SweepParams 
         }
     }
     if (p.skip_barrier_cta0 && c == 0) return;  // test hook: the others' waits must run out
-    if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns)) return;
+    if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns, p.cluster)) return;
 
     double T = 1.0;
     if (tid == 0 && !BF) {
@@ -391,7 +391,7 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_kernel(const SweepParams 
             if (edges_done) atomicAdd((unsigned long long*)&sb->edges, (unsigned long long)edges_done);
             edges_done = 0;
         }
-        if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns)) return;
+        if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns, p.cluster)) return;
         if (tid == 0) {
             sh.res = ld_relaxed_f64(&sb->acc_res[slot]);
             sh.gprev = ld_relaxed_f64(&sb->acc_g[slot]);
@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_kernel(const SweepParams 
             if (!dense) {
                 mark_out_tiles(p.fr_chg + row_lo, sh.nchg, p.fr_orow, p.fr_otile, p.fr_oend, p.fr_act, it, warp,
                                NWARP);
-                if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns)) return;
+                if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns, p.cluster)) return;
             }
         }
     }
@@ -481,6 +481,32 @@ int set_l1_carveout(const void* k, int device, int threads, size_t static_smem, 
         DAG_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, pct));
     }
     if (pct_out) *pct_out = pct;
+    return DAG_OK;
+}
+
+int launch_sweep_grid(const void* k, int nb, size_t dyn, SweepParams& p, cudaStream_t s)
+{
+    // (the test hooks leave a CTA out of a barrier: those solves wait in memory, with a limit)
+    p.cluster = nb <= CLUSTER_MAX && !p.skip_barrier_cta0 && !p.stall_fill ? 1 : 0;
+    void* args[] = {(void*)&p};
+    if (p.cluster) {
+        if (nb > 8) DAG_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = (unsigned)nb;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(nb);
+        cfg.blockDim = dim3(NT);
+        cfg.dynamicSmemBytes = dyn;
+        cfg.stream = s;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        if (cudaLaunchKernelExC(&cfg, k, args) == cudaSuccess) return DAG_OK;
+        cudaGetLastError();  // the cluster does not fit (a device shared in smaller parts): nothing was enqueued
+        p.cluster = 0;
+    }
+    DAG_CUDA(cudaLaunchCooperativeKernel(k, dim3(nb), dim3(NT), args, dyn, s));
     return DAG_OK;
 }
 
@@ -691,10 +717,10 @@ int launch_sweep(dag_plan* plan, int mode, int variant, int delta, SweepParams& 
             return set_error(DAG_ERR_INVALID, "graph, weight and state arrays must be 16-byte aligned");
     DAG_CUDA(cudaMemsetAsync(plan->sync, 0, sizeof(SyncBlock), s));
     KernelFn k = kernel_for(mode, variant, p.frontier != 0);
-    void* args[] = {(void*)&p};
     size_t dyn = sweep_ring_bytes(mode, variant) + ((variant == DAG_DELAYED) ? (size_t)cap * 4 : 0);
     DAG_CUDA(cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
-    DAG_CUDA(cudaLaunchCooperativeKernel((const void*)k, dim3(nb), dim3(NT), args, dyn, s));
+    rc = launch_sweep_grid((const void*)k, nb, dyn, p, s);
+    if (rc) return rc;
     *out_nblocks = nb;
     return DAG_OK;
 }

@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_tma_kernel(const SweepPar
         }
     }
     if (p.skip_barrier_cta0 && c == 0) return;  // test hook: the others' waits must run out
-    if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns)) return;
+    if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns, p.cluster)) return;
 
     double T = 1.0;
     if (tid == 0 && !BF) {
@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_tma_kernel(const SweepPar
             if (e) atomicAdd((unsigned long long*)&sb->edges, (unsigned long long)e);
             edges_done = 0;
         }
-        if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns)) return;
+        if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns, p.cluster)) return;
         if (tid == 0) {
             sh.res = ld_relaxed_f64(&sb->acc_res[slot]);
             if (FRONTIER || MODE == MODE_ADJ) sh.gprev = ld_relaxed_f64(&sb->acc_g[slot]);
@@ -530,9 +530,9 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_tma_kernel(const SweepPar
                 else
                     mark_out_tiles(p.fr_chg + row_lo, sh.nchg, p.fr_orow, p.fr_otile, p.fr_oend, p.fr_act, it,
                                    warp, NWARP);
-                if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns)) return;
+                if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns, p.cluster)) return;
                 publish_tiles(sh, p.fr_act, it + 1, tile_lo, tile_hi, p.fr_glist, &sb->fr_cnt[(it + 1) % 3]);
-                if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns)) return;
+                if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns, p.cluster)) return;
             }
         }
     }

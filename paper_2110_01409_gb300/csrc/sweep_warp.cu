@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_kernel(const SweepP
         }
     }
     if (p.skip_barrier_cta0 && c == 0) return;  // test hook: the others' waits must run out
-    if (!p.shard && !grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns)) return;
+    if (!p.shard && !grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns, p.cluster)) return;
 
     double T = 1.0;
     if (tid == 0 && !BF) {
@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_kernel(const SweepP
         // -------- end of sweep: residual, barrier, stopping rule --------
         __syncwarp();  // (block_add uses the warp's val)
         block_add(sh, res_part, &sb->acc_res[slot], g_part, ((SYNC || MODE == MODE_ADJ) && !BF) ? &sb->acc_g[slot] : nullptr);
-        if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns)) return;
+        if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns, p.cluster)) return;
         if (tid == 0) {
             sh.res = ld_relaxed_f64(&sb->acc_res[slot]);
             sh.gprev = ld_relaxed_f64(&sb->acc_g[slot]);
@@ -378,7 +378,7 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_ordered_kernel(const Swe
         }
     }
     if (p.skip_barrier_cta0 && c == 0) return;  // test hook: the others' waits must run out
-    if (!grid_barrier_call(sb, p.nblocks, bar_target, p.timeout_ns)) return;
+    if (!grid_barrier_call(sb, p.nblocks, bar_target, p.timeout_ns, p.cluster)) return;
 
     double T_tot = 1.0;
     if (tid == 0 && !BF) {
@@ -541,7 +541,7 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_ordered_kernel(const Swe
         // -------- end of sweep: residual, barrier, stopping rule --------
         __syncwarp();  // (block_add uses the warp's val)
         block_add(sh, res_part, &sb->acc_res[slot], g_part, MODE == MODE_ADJ ? &sb->acc_g[slot] : nullptr);
-        if (!grid_barrier_call(sb, p.nblocks, bar_target, p.timeout_ns)) return;
+        if (!grid_barrier_call(sb, p.nblocks, bar_target, p.timeout_ns, p.cluster)) return;
         if (tid == 0) {
             sh.res = ld_relaxed_f64(&sb->acc_res[slot]);
             if (MODE == MODE_ADJ) sh.gprev = ld_relaxed_f64(&sb->acc_g[slot]);
@@ -766,8 +766,8 @@ int launch_warp_sweep(dag_plan* plan, int mode, int variant, int delta, SweepPar
     const void* k = warp_kernel(kind, mode, variant, plan->warp_ipt, ordered);
     const size_t dyn = (size_t)WWARPS * (size_t)cap * 4;
     DAG_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
-    void* args[] = {(void*)&p};
-    DAG_CUDA(cudaLaunchCooperativeKernel(k, dim3(nb), dim3(NT), args, dyn, s));
+    rc = launch_sweep_grid(k, nb, dyn, p, s);
+    if (rc) return rc;
     *out_nblocks = nb * WWARPS;
     return DAG_OK;
 }

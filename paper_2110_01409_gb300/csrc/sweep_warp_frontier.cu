@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_frontier_kernel(con
         init_values<MODE>(p, X, unused_n, unused_t);
     }
     if (p.skip_barrier_cta0 && c == 0) return;  // test hook: the others' waits must run out
-    if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns)) return;
+    if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns, p.cluster)) return;
 
     const int rmode = p.read_mode == READ_CACHED ? READ_CACHED : READ_COHERENT;
     const uint64_t pol_edge = policy_evict_first();
@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_frontier_kernel(con
         __syncwarp();  // (block_add uses the warp's val)
         block_add_count(sh, res_part, &sb->acc_res[slot], (long long)marks, &sb->acc_g[slot]);
         if (lane == 0 && edges) atomicAdd((unsigned long long*)&sb->edges, (unsigned long long)edges);
-        if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns)) return;
+        if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns, p.cluster)) return;
         if (tid == 0) {
             sh.res = ld_relaxed_f64(&sb->acc_res[slot]);
             sh.gprev = ld_relaxed_f64(&sb->acc_g[slot]);
@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_frontier_kernel(con
                 stamp_edge_tiles(cta_chg, own_cnt, p.fr_orow, p.fr_otile, p.fr_act, 0, wl, WWARPS, lane);
             else
                 stamp_edge_tiles(own_chg, own_cnt, p.fr_orow, p.fr_otile, p.fr_act, 0, 0, 1, lane);
-            if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns)) return;
+            if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns, p.cluster)) return;
         }
     }
 

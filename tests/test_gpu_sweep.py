@@ -354,3 +354,28 @@ def test_last_status_copied_on_the_device(dag):
     got = st_dev.cpu().numpy()
     assert got[0, 0] == 0 and got[0, 1] == 1 and got[0, 2] > 2
     assert got[1, 0] == 0 and got[1, 1] == 0 and got[1, 2] == 2
+
+
+@pytest.mark.parametrize("tiles", [1, 2, 8, 9, 16, 17])
+@pytest.mark.parametrize("variant,delta,reads", [("sync", 0, "refresh"), ("async", 0, "refresh"),
+                                                 ("async", 0, "ordered"), ("sync", 0, "warp")])
+def test_grids_around_one_cluster(dag, tiles, variant, delta, reads):
+    # exactly `tiles` CTA tiles (or as many CTAs of warps): one cluster up to 16 CTAs (8 is the portable size),
+    # the memory barrier above
+    per = 1792 if reads == "refresh" else 8 * 32 * 5
+    n = 12 * tiles + 60  # so many vertices that so many distinct edges exist
+    m = tiles * per - n
+    rng = np.random.default_rng(tiles)
+    k = rng.permutation(n * (n - 1))[:m]
+    s, t = k // (n - 1), k % (n - 1)
+    g = _from_edges(n, s, t + (t >= s))
+    assert g.m == m
+    plan = _plan(dag, g)
+    rstar = oracle.dense_pagerank(g, 0.85)
+    r, st = dag.pagerank(plan, 0.85, 1e-6, variant, delta, reads=reads)
+    assert st["converged"] and _l1(r, rstar) <= 1e-5, st
+    w = I.weights_u32(g, 1)
+    ref = oracle.dijkstra(g, w, 0)
+    for rd in (reads, "frontier") if reads == "refresh" else (reads,):
+        d, st = dag.sssp(plan, 0, _w_dev(w), variant, delta, reads=rd)
+        assert st["converged"] and np.array_equal(_u32(d), ref), rd

@@ -181,3 +181,21 @@ def test_ordered_barrier_timeout_leaves_context_usable(dag):
     assert ei.value.code == dag.ERR_BARRIER_TIMEOUT
     r, st = dag.pagerank(plan, 0.85, 1e-6, "async", 0, reads="ordered")
     assert st["converged"] and _l1(r, oracle.pagerank_fixed_point(g, 0.85)) <= 1e-5
+
+
+@pytest.mark.parametrize("off", [1, 2, 3])
+@pytest.mark.parametrize("reads", ["warp", "ordered", "ordered+frontier"])
+def test_warp_edge_arrays_at_any_alignment(dag, off, reads):
+    # the edge sources come in whole 16-byte granules around a tile's own, wherever the array starts; weights of one
+    # byte may start at any byte
+    g = I.rmat(11, 16, seed=5)
+    rp = torch.from_numpy(g.rowptr).cuda()
+    ci = torch.cat([torch.full((off,), -1, dtype=torch.int32), torch.from_numpy(g.colidx)]).cuda()[off:]
+    plan = dag.Plan(rp, ci)
+    w = I.weights_u32(g, 1) & 0xFF
+    wd = torch.cat([torch.zeros(off, dtype=torch.uint8), torch.from_numpy(w.astype(np.uint8))]).cuda()[off:]
+    d, st = dag.sssp(plan, 0, wd, "async", 0, reads=reads)
+    assert st["converged"] and np.array_equal(d.cpu().numpy().view(np.uint32), oracle.dijkstra(g, w, 0))
+    if "frontier" not in reads:
+        r, st = dag.pagerank(plan, 0.85, 1e-6, "async", 0, reads=reads)
+        assert st["converged"] and _l1(r, oracle.dense_pagerank(g, 0.85)) <= 1e-5
