@@ -19,8 +19,8 @@
 // columns) and were 5 to 30% slower.
 //
 // Measured (RMAT, against a CTA block of whole rows walked in tiles by eight warps with a barrier per tile, and a
-// warp of 32 columns for other column counts): PPR of 256 columns at 1 M vertices 66.5 -> 27.3 ms, of 20 columns at
-// 100 K vertices 7.06 -> 1.19 ms (a hub's row was one warp's), Bellman-Ford of 64 columns at 1 M vertices 24.4 -> 7.5.
+// warp of 32 columns for other column counts): PPR of 256 columns at 1 M vertices 66.5 -> 26.3 ms, of 20 columns at
+// 100 K vertices 7.06 -> 1.05 ms (a hub's row was one warp's), Bellman-Ford of 64 columns at 1 M vertices 24.4 -> 7.5.
 // Slower than that kernel on small uniform graphs of 32 columns only (3 K vertices, PPR: 165 -> 200 us).
 //
 // Bellman-Ford reads only what can lower something: chg[u] is the last sweep that lowered any of u's columns, and
@@ -120,6 +120,15 @@ constexpr int run_min_blocks(bool BF, int CH) { return CH >= 4 ? 1 : CH == 2 || 
 // 28 KB of L1: Bellman-Ford uniform 20 K 615 -> 490 us with half of it (RMAT 1 M 7.1 -> 7.5 ms).
 constexpr int run_depth(int LPR, int CH) { return CH >= 4 ? 4 : CH == 2 ? 8 : LPR >= 16 ? 16 : 32; }
 
+// The ring's rows are as long as the lanes that hold them, so that a row that does not fill them is added up without a
+// test per chunk and with constant addresses; columns past its end hold what is there and are never stored. PPR, RMAT
+// 262 K and uniform 100 K vertices: 20 columns 2.32 -> 2.08 and 1.19 -> 1.05 ms, 68 columns 5.60 -> 5.01 and 2.12 ->
+// 1.92 (both with EVERY, below, half of it), 200 columns 7.80 -> 7.29 and 3.03 -> 2.85; Bellman-Ford 500 columns 14.7
+// -> 11.8 and 9.2 -> 7.5. Not Bellman-Ford of 65 to 128 columns, where the longer ring takes L1 from the last-change
+// bytes (100 columns, RMAT: 3.71 -> 3.93). EVERY on rows of several chunks lost: 136 columns 7.0 -> 9.6 ms, as most
+// lanes of the last chunk fetch one address.
+constexpr bool run_padded(bool BF, int LPR, int CH) { return !BF || LPR < 32 || CH > 1; }
+
 // LPR lanes hold a row (four columns per lane and chunk), CH chunks per lane (more than one only with LPR = 32);
 // WHOLE: the row fills them all, so its length is a constant.
 template <bool BF, int LPR, int CH, bool WHOLE>
@@ -129,9 +138,11 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
     constexpr int GRP = 32 / LPR;          // in-edges a warp adds at a time
     constexpr int RW = BF ? 1 : 2;         // items at a row end
     constexpr int D = run_depth(LPR, CH), G = D / 2;
+    constexpr bool PAD = run_padded(BF, LPR, CH), EVERY = !BF && CH == 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
 
     const int B = p.B, S = WHOLE ? 4 * LPR * CH : p.stride, NCH = S >> 2;
+    const int SR = PAD ? 4 * LPR * CH : S;  // values between fetched rows
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int grp = lane / LPR, lr = lane % LPR;
     const bool sync = p.sync != 0;
@@ -145,9 +156,9 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
     int* s_run = s_last + S;                                      // [S] 1: the column still runs
     float* s_live = (float*)(s_run + S);                          // [S] PPR: the CTA's change of the live mass
     int* s_list = (int*)(s_live + (BF ? 0 : S));                                      // [RUN_WARPS][2][2][32] items: vertex, weight
-    uint32_t* s_ring = (uint32_t*)(s_list + RUN_WARPS * 128);     // [RUN_WARPS][D][S] fetched rows
+    uint32_t* s_ring = (uint32_t*)(s_list + RUN_WARPS * 128);     // [RUN_WARPS][D][SR] fetched rows
     int* list = s_list + warp * 128;
-    uint32_t* ring = s_ring + (size_t)warp * D * S;
+    uint32_t* ring = s_ring + (size_t)warp * D * SR;
     uint32_t* head_sum = s_head + warp * S;
     uint32_t* fold = (uint32_t*)s_red + warp * S;  // PPR, during the sweep: the folded part of the row in progress
     const uint32_t ring_at = smem_addr(ring);
@@ -158,6 +169,8 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
     // the columns of this lane's chunk q: 4 (lr + 32 q) .. + 3
     auto col0 = [&](int q) { return 4 * (lr + 32 * q); };
     auto has = [&](int q) { return WHOLE || lr + 32 * q < NCH; };
+    // EVERY: a lane without columns copies the row's last four too (and never stores them), which saves the branch
+    auto from = [&](int q) { return !EVERY || has(q) ? col0(q) : S - 4; };
 
     // per-column sums of the CTA's warps (group 0's lanes hold them), added in a fixed order, one FP64 atomic each
     auto cta_sum = [&](const float (&part)[CH][4], double* dst, double* dst2) {
@@ -559,7 +572,7 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
         // copies of batch b of a stage into ring half `half`
         auto fetch = [&](const RunStage& st, int lb, int b, int half) {
             const int* lv = list + lb * 64 + b * G;
-            const uint32_t at = ring_at + (uint32_t)(half * G * S + 4 * lr) * 4u;
+            const uint32_t at = ring_at + (uint32_t)(half * G * SR + 4 * lr) * 4u;
             const int have = st.cnt - b * G;
             const unsigned tele = BF ? 0u : st.fin >> (b * G);
 #pragma unroll
@@ -567,17 +580,17 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
                 const int k = u * GRP + grp;
                 if (k >= have || (G < GRP && k >= G)) continue;
                 const int v = lv[k];
-                const uint32_t dst = at + (uint32_t)(k * S) * 4u;
+                const uint32_t dst = at + (uint32_t)(k * SR) * 4u;
                 if (BF || !((tele >> k) & 1u)) {
-                    const uint32_t* x = xin + (size_t)v * S + 4 * lr;
+                    const uint32_t* x = xin + (size_t)v * S;
 #pragma unroll
                     for (int q = 0; q < CH; ++q)
-                        if (has(q)) cp16(dst + 512u * q, x + 128 * q);
+                        if (EVERY || has(q)) cp16(dst + 512u * q, x + from(q));
                 } else if (p.v16) {
-                    const float* x = p.V + (size_t)v * B + 4 * lr;
+                    const float* x = p.V + (size_t)v * B;
 #pragma unroll
                     for (int q = 0; q < CH; ++q)
-                        if (has(q)) cp16(dst + 512u * q, x + 128 * q);
+                        if (EVERY || has(q)) cp16(dst + 512u * q, x + from(q));
                 } else {
 #pragma unroll
                     for (int q = 0; q < CH; ++q)
@@ -591,13 +604,13 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
         // batch b of a stage from ring half `half`
         auto consume = [&](const RunStage& st, int lb, int b, int half) {
             const int* lv = list + lb * 64 + b * G;
-            const uint32_t* rows = ring + half * G * S + 4 * lr;
+            const uint32_t* rows = ring + half * G * SR + 4 * lr;
             auto add = [&](int k) {
                 const uint32_t wt = BF ? (uint32_t)lv[32 + k] : 0u;
 #pragma unroll
                 for (int q = 0; q < CH; ++q) {
-                    if (!has(q)) continue;
-                    const uint4 x = *(const uint4*)(rows + k * S + 128 * q);
+                    if (!PAD && !has(q)) continue;
+                    const uint4 x = *(const uint4*)(rows + k * SR + 128 * q);
                     acc[q][0] = comb<BF>(acc[q][0], BF ? relax_w(x.x, wt) : x.x);
                     acc[q][1] = comb<BF>(acc[q][1], BF ? relax_w(x.y, wt) : x.y);
                     acc[q][2] = comb<BF>(acc[q][2], BF ? relax_w(x.z, wt) : x.z);
@@ -626,7 +639,7 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
 #pragma unroll
                 for (int q = 0; q < CH; ++q) {
                     x[q] = make_uint4(0u, 0u, 0u, 0u);
-                    if (has(q)) x[q] = *(const uint4*)(rows + e1 * S + 128 * q);
+                    if (PAD || has(q)) x[q] = *(const uint4*)(rows + e1 * SR + 128 * q);
                 }
                 if (!BF && ((old >> e1) & 1u)) {
 #pragma unroll
@@ -838,8 +851,9 @@ size_t run_smem_bytes(bool is_bf, int B)
 {
     const size_t S = (size_t)((B + 3) & ~3);
     const int k = run_shape(B), depth = run_depth(k < 5 ? 1 << k : 32, k > 5 ? 1 << (k - 5) : 1);
+    const size_t SR = run_padded(is_bf, k < 5 ? 1 << k : 32, k > 5 ? 1 << (k - 5) : 1) ? (size_t)4 << k : S;
     return (is_bf ? 0 : 2 * S * 8 + S * 4) + 2 * RUN_WARPS * S * 4 + 2 * S * 4 + RUN_WARPS * 128 * 4 +
-           (size_t)RUN_WARPS * depth * S * 4;
+           (size_t)RUN_WARPS * depth * SR * 4;
 }
 
 // PPR: two items to fetch, an update and a store, against an in-edge's one addition, which costs the less the fewer
