@@ -479,9 +479,9 @@ constexpr int RUN_MIN_ITEMS = 16;
 constexpr int RUN_ITEMS = 1024;
 constexpr int RUN_ITEMS_WIDE = 256;
 
-int launch_batched(dag_plan* plan, int is_bf, int variant, int delta, int max_iters, int B, float d, double tol,
-                   const void* V_or_src, const uint32_t* w, void* out, int* iters, dag_batch_stats* st,
-                   cudaStream_t s)
+static int launch_on(bool runs, dag_plan* plan, int is_bf, int variant, int delta, int max_iters, int B, float d,
+                     double tol, const void* V_or_src, const uint32_t* w, void* out, int* iters, dag_batch_stats* st,
+                     cudaStream_t s)
 {
     const int n = plan->n;
     const int W = (B + 31) / 32;
@@ -498,7 +498,6 @@ int launch_batched(dag_plan* plan, int is_bf, int variant, int delta, int max_it
     size_t dyn = (size_t)(2 * TILE + 1 + (is_bf ? TILE : 0)) * 4 + (size_t)W * dl * 32 * 4;
     BKernel k = bkernel_for(is_bf, variant);
     int threads_launch = threads;
-    const bool runs = plan->batched_wide && variant != DAG_DELAYED;
     if (runs) {
         k = run_kernel_for(is_bf != 0, B);
         threads_launch = NT;
@@ -668,6 +667,19 @@ int launch_batched(dag_plan* plan, int is_bf, int variant, int delta, int max_it
     st->graph = replayed ? 1 : 0;
     if (rc2 == DAG_ERR_BARRIER_TIMEOUT) set_error(rc2, "grid barrier wait ran out of time");
     return rc2;
+}
+
+// Runs of the merge path but for the delayed form; where their scratch (partials, a padded copy of rows that are not
+// whole 16-byte chunks) does not fit on the device, the 32-column kernel, whose in-place forms take none.
+int launch_batched(dag_plan* plan, int is_bf, int variant, int delta, int max_iters, int B, float d, double tol,
+                   const void* V_or_src, const uint32_t* w, void* out, int* iters, dag_batch_stats* st,
+                   cudaStream_t s)
+{
+    const bool runs = plan->batched_wide && variant != DAG_DELAYED;
+    const int rc = launch_on(runs, plan, is_bf, variant, delta, max_iters, B, d, tol, V_or_src, w, out, iters, st, s);
+    if (!runs || rc != DAG_ERR_NOMEM) return rc;
+    cudaGetLastError();  // the allocation's
+    return launch_on(false, plan, is_bf, variant, delta, max_iters, B, d, tol, V_or_src, w, out, iters, st, s);
 }
 
 }  // namespace dag
