@@ -208,7 +208,7 @@ struct dag_plan {
     int* nw_hubs = nullptr;   // sources of more than NW_HUB out-edges (summed by a whole block)
     int nw_nhubs = 0;
     void* grad_coef = nullptr;  // [n] float2 (d r_u / s_u, (M^T lambda)_u) of the edge gradients, first use
-    std::map<long long, dag::Partition> parts;  // key: nblocks | row_cap << 32
+    std::map<long long, dag::Partition> parts;  // key: nblocks | row_cap << 32 | row weight << 44
     std::map<std::tuple<int, int, int, int, int, int>, dag::Shape> shapes;  // see sweep_shape, warp_shape
     std::map<std::pair<const void*, size_t>, std::pair<int, int>> batched_fit;  // (kernel, dyn) -> CTAs per SM, carveout
     cudaEvent_t ev[2] = {nullptr, nullptr};  // around a solve whose time is asked for
@@ -234,7 +234,7 @@ int cuda_check(cudaError_t e, const char* what);
     } while (0)
 
 // plan.cu
-int get_partition(dag_plan* plan, int nblocks, Partition** out, cudaStream_t s, int row_cap);
+int get_partition(dag_plan* plan, int nblocks, Partition** out, cudaStream_t s, int row_cap, int row_w = 1);
 
 // The frontier maps of a partition (and the plan's out-CSR row pointers), built once.
 int frontier_maps(dag_plan* plan, Partition* part, cudaStream_t s, bool with_end = true);

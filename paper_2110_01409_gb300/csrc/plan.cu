@@ -221,10 +221,14 @@ __global__ void k_tile_end(int tiles, int n, long long m, int* tile_row, int* ti
     tile_nz[tiles] = (int)m;
 }
 
-int get_partition(dag_plan* plan, int P, Partition** out, cudaStream_t s, int row_cap)
+int get_partition(dag_plan* plan, int P, Partition** out, cudaStream_t s, int row_cap, int row_w)
 {
     if (row_cap >= TILE) row_cap = 0;  // a tile never holds more than TILE rows
-    const long long key = (long long)P | ((long long)row_cap << 32);
+    // Row-capped tiles cost a tile per row_cap rows even where rows have no
+    // edges, so their blocks weigh each row at least ceil(TILE / row_cap): a
+    // block's tile count then follows its weight, as it does uncapped.
+    if (row_cap > 0) row_w = std::max(row_w, (TILE + row_cap - 1) / row_cap);
+    const long long key = (long long)P | ((long long)row_cap << 32) | ((long long)row_w << 44);
     auto it = plan->parts.find(key);
     if (it != plan->parts.end()) { *out = &it->second; return DAG_OK; }
     Partition part;
@@ -235,10 +239,6 @@ int get_partition(dag_plan* plan, int P, Partition** out, cudaStream_t s, int ro
     DAG_CUDA(dev_alloc(&part.cta_row, (P + 1) * sizeof(int)));
     DAG_CUDA(dev_alloc(&part.cta_tile, (P + 1) * sizeof(int)));
     DAG_CUDA(dev_alloc(&mr_dev, sizeof(int)));
-    // Row-capped tiles cost a tile per row_cap rows even where rows have no
-    // edges, so their blocks weigh each row ceil(TILE / row_cap) instead of 1:
-    // a block's tile count then follows its weight, as it does uncapped.
-    const int row_w = row_cap > 0 ? (TILE + row_cap - 1) / row_cap : 1;
     long long total = (long long)row_w * plan->n + plan->m;
     k_cta_rows<<<(P + 1 + 255) / 256, 256, 0, s>>>(plan->rowptr, plan->n, total, P, part.cta_row, row_w);
     if (row_cap > 0) {
@@ -424,7 +424,10 @@ int get_batch_runs(dag_plan* plan, int W, int row_w, Partition** out, cudaStream
     Partition part;
     part.nblocks = W;
     DAG_CUDA(dev_alloc(&part.cta_row, (W + 1) * sizeof(int)));
-    DAG_CUDA(dev_alloc(&part.cta_tile, (W + 1) * sizeof(int)));
+    if (const cudaError_t e = dev_alloc(&part.cta_tile, (W + 1) * sizeof(int)); e != cudaSuccess) {
+        dev_free(part.cta_row);
+        return cuda_check(e, "batched runs");
+    }
     k_batch_runs<<<(W + 1 + 255) / 256, 256, 0, s>>>(plan->rowptr, plan->n, (long long)row_w * plan->n + plan->m, row_w,
                                                      W, part.cta_row, part.cta_tile);
     DAG_CUDA(cudaGetLastError());

@@ -632,6 +632,20 @@ int settle_shape(dag_plan* plan, int mode, int variant, int delta,
     return DAG_OK;
 }
 
+// A row's weight beside its in-edges in the cuts of the CTAs' blocks (Sec. III-A weighs in-degree + 1, for a CPU
+// thread's work; the tiles stay equal shares of the merge path). A tile of rows without in-edges costs a CTA two to
+// three times one of edges, and RMAT's lie together, so the sweeps waited for the blocks that hold them. Weights 1, 2,
+// 3, 5, RMAT, 4 M vertices, ms: PageRank sync 7.71, 6.02, 5.94, 6.22 (1 M: 1.62, 1.33, 1.25, 1.35), delta 4096 9.54,
+// 7.17, 6.93, 7.18, async 4.50, 3.82, 4.24, 4.33; Bellman-Ford async 3.82, 3.57, 3.72, 4.00, with the frontier 3.74,
+// 2.77, 2.86, 3.07. Graphs without skew do not move. Synchronous Bellman-Ford keeps 1 (4.49 against 4.30): the edges
+// that its frontier runs, a result, are those of Sec. III-A's blocks.
+static int cta_row_weight(int mode, int variant)
+{
+    const bool bf = mode == MODE_BF || mode == MODE_BF8;
+    if (bf && variant == DAG_SYNC) return 1;
+    return bf || variant == DAG_ASYNC ? 2 : 3;
+}
+
 // Launch shape and the plan's cached partition for it (a delayed sweep with
 // delta below a tile's items gets tiles of at most delta rows).
 int sweep_shape(dag_plan* plan, int mode, int variant, int delta, int* nb_out, int* cap_out, Partition** part_out,
@@ -651,7 +665,7 @@ int sweep_shape(dag_plan* plan, int mode, int variant, int delta, int* nb_out, i
     Partition* part = nullptr;
     int clamped = 0;
     auto build = [&](int nb, int* max_rows) {
-        const int rc = get_partition(plan, nb, &part, s, delayed_row_cap(variant, delta));
+        const int rc = get_partition(plan, nb, &part, s, delayed_row_cap(variant, delta), cta_row_weight(mode, variant));
         if (rc == DAG_OK) *max_rows = part->max_rows;
         return rc;
     };

@@ -6,7 +6,7 @@
 //  * worker = one warp. The merge path of the whole graph (rows and in-edges
 //    in vertex order, Merrill & Garland) is cut into warp tiles of WTILE items
 //    and every worker takes a run of consecutive tiles of equal weight
-//    (in-degree + WARP_ROW_WEIGHT per row, Sec. III-A's balance with a row's
+//    (in-degree + 2 or 3 per row, Sec. III-A's balance with a row's
 //    cost on this machine) and owns the rows whose end item lies in its run (contiguous in vertex order). A row whose
 //    in-edges span two runs (a hub, or a cut inside a row) is owned by the run
 //    that ends it; the earlier runs' partial sums reach it at the end of the
@@ -616,8 +616,13 @@ static const void* warp_kernel(int kind, int mode, int variant, int ipt, bool or
 // rows without in-edges lie together (RMAT: half the rows), runs of equal item counts held up to 6,600 rows against a
 // mean of 430 and the sweep waited for them. Weights 1, 2, 3, 4, RMAT, ms: CTA-ordered frontier Bellman-Ford (4 M
 // vertices) 2.99, 2.19-2.5, 2.05-2.35, 2.3-2.55; weighted PageRank and its adjoint (2 M) 2.78 + 2.4, 2.05 + 1.9,
-// 1.95 + 1.79, 1.99 + 1.98; delayed Bellman-Ford (1 M) 1.28, 1.21, 1.15, 1.21. Graphs without skew do not move.
-constexpr int WARP_ROW_WEIGHT = 3;
+// 1.95 + 1.79, 1.99 + 1.98. Bellman-Ford on warp runs, whose edges cost more (a weight each) and rows less (no degree),
+// at 4 M, weights 1, 2, 3: sync 4.33, 3.91, 3.95, delta 256 4.41, 3.95, 4.35, async 3.87, 3.45, 3.48. Graphs without skew
+// do not move.
+static int warp_row_weight(int kind, int mode)
+{
+    return kind == WARP_RUNS && (mode == MODE_BF || mode == MODE_BF8) ? 2 : 3;
+}
 
 static int warp_shape(dag_plan* plan, int mode, int variant, int delta, int* nb_out, int* cap_out, int* clamped_out,
                       Partition** part_out, cudaStream_t s, int kind, bool ordered = false)
@@ -667,7 +672,7 @@ static int warp_shape(dag_plan* plan, int mode, int variant, int delta, int* nb_
     if (rc) return rc;
     bool settled = false;  // CTAs per SM only fall, so a few passes settle the shape
     for (int iter = 0; iter < 6 && !settled; ++iter) {
-        rc = get_warp_partition(plan, nb * WWARPS, WTILE, WARP_ROW_WEIGHT, &part, s);
+        rc = get_warp_partition(plan, nb * WWARPS, WTILE, warp_row_weight(kind, mode), &part, s);
         if (rc) return rc;
         settled = true;
         if (variant != DAG_DELAYED) break;
@@ -797,7 +802,7 @@ int sweep_rows(dag_plan* plan, int mode, int lo, int hi, SweepParams& p, double*
     int nb = per_sm * plan->num_sms;
     if (plan->worker_cap > 0) nb = std::min(nb, plan->worker_cap);
     Partition* part = nullptr;
-    int rc = get_warp_partition_range(plan, nb * WWARPS, WTILE, WARP_ROW_WEIGHT, lo, hi, &part, s);
+    int rc = get_warp_partition_range(plan, nb * WWARPS, WTILE, warp_row_weight(WARP_RUNS, mode), lo, hi, &part, s);
     if (rc) return rc;
     p.nblocks = nb;
     p.max_iters = 1;
