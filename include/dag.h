@@ -96,7 +96,9 @@ int dag_plan_destroy(dag_plan* plan);
 int dag_plan_out_degree(const dag_plan* plan, int32_t* d_outdeg, void* stream);
 
 /*
- * The static partition the sweep kernels use for `workers` CTAs (Sec. III-A):
+ * The static partition of Sec. III-A for `workers` CTAs (that of the
+ * synchronous Bellman-Ford sweeps and the access matrix; the other CTA sweeps
+ * weigh a vertex in-degree + 2 or more, by what a row's update costs a CTA):
  * h_start[p] (host, workers+1 values) is the first vertex of block p, chosen
  * so that every block carries about (n + m)/workers of the weight
  * (in-degree + 1) per vertex: h_start[p] = min { v : v + rowptr[v] >=
@@ -168,7 +170,7 @@ int dag_plan_set_worker_cap(dag_plan* plan, int32_t max_workers);
  * worker of Sec. III-A is one warp instead of one CTA. The merge path of the
  * whole graph (rows and in-edges in vertex order) is cut into tiles of
  * dag_warp_tile_items(plan) items and each warp takes a run of them, so that
- * workers are balanced by in-degree + 3 per row (Sec. III-A's in-degree + 1,
+ * workers are balanced by in-degree + 2 or 3 per row (Sec. III-A's in-degree + 1,
  * with what a row's update costs a warp beside an in-edge); a warp owns the
  * rows that end in its run, and a row whose in-edges span several runs gets
  * the earlier runs' partial sums at the end of the sweep. delta counts rows

@@ -60,7 +60,7 @@ static int bits_for(int n)
 
 // ---------------------------------------------------------------------------
 // Partition: block p starts at min { v : v + rowptr[v] >= ceil(p (n+m) / P) }
-// (every vertex weighs in-degree + 1), then each block is cut into merge-path
+// (every vertex weighs in-degree + 1, or + row_w), then each block is cut into merge-path
 // tiles of TILE items; a tile's start is (rows ended before it, edges before it).
 // ---------------------------------------------------------------------------
 // row_w: weight of a row beside its in-edges (1: Sec. III-A's in-degree + 1;

@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_kernel(const SweepParams 
 
         // Software pipeline: while tile t is walked, tile t+1's edge stream,
         // row ends and old values are in flight (issued after barrier A of t)
-        // and its gathers too (issued before barrier C of t).
+        // and its gathers too (issued after barrier B of t).
         Stage<MODE> nx;
         if (ntl > 0) {
             stage_issue<MODE>(nx, p, tile_at(0), tid, pol_edge, pol_vertex);

@@ -20,7 +20,7 @@
 //  * one grid barrier per iteration (Sec. I) and the stopping rules of Sec. IV.
 //
 // Why warps: the CTA-tile kernels (sweep.cu, sweep_tma.cu) stop all eight
-// warps at three barriers per 1,792-item tile, so each tile waits for its
+// warps at two barriers per 1,792-item tile, so each tile waits for its
 // slowest gather; here each warp sums its own 224-item tiles with a
 // shuffle-only segmented scan, copies edge sources two tiles ahead (cp.async)
 // and issues the next tile's gathers before the current one's sums or after
