@@ -224,10 +224,6 @@ __global__ void k_tile_end(int tiles, int n, long long m, int* tile_row, int* ti
 int get_partition(dag_plan* plan, int P, Partition** out, cudaStream_t s, int row_cap, int row_w)
 {
     if (row_cap >= TILE) row_cap = 0;  // a tile never holds more than TILE rows
-    // Row-capped tiles cost a tile per row_cap rows even where rows have no
-    // edges, so their blocks weigh each row at least ceil(TILE / row_cap): a
-    // block's tile count then follows its weight, as it does uncapped.
-    if (row_cap > 0) row_w = std::max(row_w, (TILE + row_cap - 1) / row_cap);
     const long long key = (long long)P | ((long long)row_cap << 32) | ((long long)row_w << 44);
     auto it = plan->parts.find(key);
     if (it != plan->parts.end()) { *out = &it->second; return DAG_OK; }

@@ -572,6 +572,15 @@ int max_workers(dag_plan* plan, int mode, int variant, int buf_cap_elems, int* o
     return DAG_OK;
 }
 
+// A row's items in tiles of at most cap rows (0: as many as fit): a capped tile of rows without edges counts as a full one.
+static int tile_row_weight(int cap) { return cap > 0 && cap < TILE ? (TILE + cap - 1) / cap : 1; }
+// Tiles of the plan's merge path, two at least (so that a barrier has someone to wait for).
+static long long path_tiles(const dag_plan* plan, int cap)
+{
+    return std::max(2LL, ((long long)tile_row_weight(cap) * plan->n + plan->m + TILE - 1) / TILE);
+}
+
+
 // Launch shape of a sweep: CTA count and delay-buffer capacity. A delayed
 // sweep's buffer holds at most min(delta - 1 + TILE, rows of the largest block)
 // values (a flush empties it once it reaches delta after a tile), and at most
@@ -591,9 +600,7 @@ int settle_shape(dag_plan* plan, int mode, int variant, int delta,
         // A small graph's sweep is its grid barrier: one CTA per tile (two at least, so that a barrier has someone to
         // wait for). Above half the resident CTAs the SMs are better filled evenly (banded, 60 K vertices: 568 CTAs of
         // a tile each 447 us, 608 of a little less 424).
-        const int cap = delayed_row_cap(variant, delta);
-        const long long row_w = cap > 0 ? (TILE + cap - 1) / cap : 1;
-        const long long tiles = std::max(2LL, (row_w * plan->n + plan->m + TILE - 1) / TILE);
+        const long long tiles = path_tiles(plan, delayed_row_cap(variant, delta));
         if (2 * tiles <= nb) nb = (int)tiles;
     }
     if (plan->worker_cap > 0 && nb > plan->worker_cap) nb = plan->worker_cap;
@@ -639,11 +646,20 @@ int settle_shape(dag_plan* plan, int mode, int variant, int delta,
 // 7.17, 6.93, 7.18, async 4.50, 3.82, 4.24, 4.33; Bellman-Ford async 3.82, 3.57, 3.72, 4.00, with the frontier 3.74,
 // 2.77, 2.86, 3.07. Graphs without skew do not move. Synchronous Bellman-Ford keeps 1 (4.49 against 4.30): the edges
 // that its frontier runs, a result, are those of Sec. III-A's blocks.
-static int cta_row_weight(int mode, int variant)
+// Tiles of at most cap rows (delta below a tile's items) come one per cap rows even where rows have no edges, so a row
+// there weighs k = ceil(TILE / cap) for the tile, and for PageRank 2 more as above; a capped tile of Bellman-Ford's rows
+// costs three quarters of one of edges. Weights k, 1.25 k, 1.5 k, PageRank: delta 256 (k = 7) 6.46, 6.17, 6.81, delta 600
+// (3) 6.88, 5.95, 5.71, delta 32 (56) 13.0, 14.3, 15.7; 0.5 k, 0.75 k, 0.85 k, k, Bellman-Ford: delta 32 10.96, 11.08,
+// 12.05, 12.89 (0.5 M vertices 1.61, 1.67, 1.51, 2.08), delta 256 4.93, 4.84, 5.06, 5.35.
+// A grid of a CTA or more per tile takes k, so that blocks are the tiles it was sized for (Bellman-Ford, 1,000 vertices,
+// delta 32: 113 us a call, 129 with two tiles in some blocks).
+static int cta_row_weight(const dag_plan* plan, int mode, int variant, int cap, int nb)
 {
     const bool bf = mode == MODE_BF || mode == MODE_BF8;
-    if (bf && variant == DAG_SYNC) return 1;
-    return bf || variant == DAG_ASYNC ? 2 : 3;
+    const int k = tile_row_weight(cap);
+    if (nb >= path_tiles(plan, cap)) return k;
+    if (bf) return variant == DAG_SYNC ? 1 : std::max(2, (3 * k + 3) / 4);
+    return variant == DAG_ASYNC ? 2 : k + 2;
 }
 
 // Launch shape and the plan's cached partition for it (a delayed sweep with
@@ -665,7 +681,8 @@ int sweep_shape(dag_plan* plan, int mode, int variant, int delta, int* nb_out, i
     Partition* part = nullptr;
     int clamped = 0;
     auto build = [&](int nb, int* max_rows) {
-        const int rc = get_partition(plan, nb, &part, s, delayed_row_cap(variant, delta), cta_row_weight(mode, variant));
+        const int cap = delayed_row_cap(variant, delta);
+        const int rc = get_partition(plan, nb, &part, s, cap, cta_row_weight(plan, mode, variant, cap, nb));
         if (rc == DAG_OK) *max_rows = part->max_rows;
         return rc;
     };
