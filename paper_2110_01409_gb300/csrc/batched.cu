@@ -504,7 +504,8 @@ static int launch_on(bool runs, dag_plan* plan, int is_bf, int variant, int delt
         dyn = run_smem_bytes(is_bf != 0, B);
     }
     int per_sm = 0;
-    const auto fit = plan->batched_fit.find({(const void*)k, dyn});
+    const auto fit_key = std::make_tuple((const void*)k, threads_launch, dyn);
+    const auto fit = plan->batched_fit.find(fit_key);
     if (fit != plan->batched_fit.end()) {
         per_sm = fit->second.first;
         Shape how;
@@ -528,7 +529,7 @@ static int launch_on(bool runs, dag_plan* plan, int is_bf, int variant, int delt
         const int rc =
             set_l1_carveout((const void*)k, plan->device, threads_launch, fa.sharedSizeBytes, dyn, per_sm, &pct);
         if (rc) return rc;
-        plan->batched_fit[{(const void*)k, dyn}] = {per_sm, pct};
+        plan->batched_fit[fit_key] = {per_sm, pct};
     }
     int nb = per_sm * plan->num_sms;
     if (plan->worker_cap > 0 && nb > plan->worker_cap) nb = plan->worker_cap;

@@ -210,7 +210,8 @@ struct dag_plan {
     void* grad_coef = nullptr;  // [n] float2 (d r_u / s_u, (M^T lambda)_u) of the edge gradients, first use
     std::map<long long, dag::Partition> parts;  // key: nblocks | row_cap << 32 | row weight << 44
     std::map<std::tuple<int, int, int, int, int, int>, dag::Shape> shapes;  // see sweep_shape, warp_shape
-    std::map<std::pair<const void*, size_t>, std::pair<int, int>> batched_fit;  // (kernel, dyn) -> CTAs per SM, carveout
+    // (kernel, threads per CTA, dynamic shared memory) -> CTAs per SM, carveout
+    std::map<std::tuple<const void*, int, size_t>, std::pair<int, int>> batched_fit;
     cudaEvent_t ev[2] = {nullptr, nullptr};  // around a solve whose time is asked for
     std::map<std::tuple<int, int, int, int>, dag::Partition> range_parts;  // (warps, tile, lo, hi)
     // batched workspace (grown on demand)

@@ -283,3 +283,26 @@ def test_runs_long_path_and_sweep_limit(dag, variant):
         assert iters.cpu().tolist() == [600, 301, 600]
         _, _, st = dag.sssp_batched(plan, src, w, variant, 0, max_iters=5)
         assert not st["converged"] and st["sweeps"] == 5
+
+
+@pytest.mark.parametrize("calls", [[("delayed", 128, 32), ("delayed", 256, 16), ("delayed", 128, 32)],
+                                   [("delayed", 32, 16), ("delayed", 512, 1)], [("sync", 8, 0), ("sync", 1024, 0)],
+                                   [("async", 8, 0), ("async", 1024, 0)]])
+def test_column_counts_of_one_kernel_and_shared_size_on_one_plan(dag, graph, calls):
+    # the 32-column kernel's CTA has a warp per 32 columns: calls whose shared memory is the same size but whose CTAs
+    # are not have grids of their own (a grid settled for the smaller CTA cannot be resident for the larger)
+    g = graph
+    plan = dag.Plan.from_graph(g, "cuda")
+    plan.set_batched_wide(False)
+    w = I.weights_u32(g, 3)
+    wd = torch.from_numpy(w.view(np.int32)).cuda()
+    for variant, B, delta in calls:
+        V = I.teleport_matrix(g.n, I.ppr_seed_sets(g.n, B, seed=2))
+        R, _, st = dag.ppr_batched(plan, torch.from_numpy(V).cuda(), 0.85, 1e-6, variant, delta)
+        assert st["converged"], st
+        rstar = oracle.pagerank_fixed_point(g, 0.85, tele=V[:, B - 1].astype(np.float64))
+        assert np.abs(R[:, B - 1].cpu().numpy().astype(np.float64) - rstar).sum() <= 1e-5
+        src = np.resize(I.sources(g, 32, seed=B), B)
+        D, _, st = dag.sssp_batched(plan, torch.from_numpy(src.view(np.int32)).cuda(), wd, variant, delta)
+        assert st["converged"]
+        assert np.array_equal(D[:, B - 1].cpu().numpy().view(np.uint32), oracle.dijkstra(g, w, int(src[B - 1])))
