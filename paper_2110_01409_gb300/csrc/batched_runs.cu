@@ -203,13 +203,15 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
                 gpart[q][e] = tpart[q][e] = 0.0f;
                 sv[q][e] = (BF && has(q) && col0(q) + e < B) ? p.src[col0(q) + e] : INF;
             }
-        for (int v = w * GRP + grp; v < p.n; v += W * GRP) {
+        for (int v0 = w * GRP; v0 < p.n; v0 += W * GRP) {  // warp-uniform: every lane takes part in the vote
+            const int v = v0 + grp;
+            const bool in = v < p.n;
             float dg = 0.0f;
-            if constexpr (!BF) dg = p.degf[v];
+            if constexpr (!BF) dg = in ? p.degf[v] : 0.0f;
             bool is_src = false;
 #pragma unroll
             for (int q = 0; q < CH; ++q) {
-                if (!has(q)) continue;
+                if (!in || !has(q)) continue;
                 uint32_t x[4];
                 if constexpr (BF) {
 #pragma unroll
@@ -240,9 +242,9 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
             }
             if constexpr (BF) {  // a source counts as changed in the sweep before the first; the value elsewhere
                                  // only costs a needless read when a solve reaches sweep 128
-                unsigned any = __ballot_sync(__activemask(), is_src);
+                unsigned any = __ballot_sync(FULL, is_src);
                 if (LPR < 32) any = (any >> (grp * LPR)) & below(LPR);
-                if (lr == 0) p.chg[v] = any ? 255 : 128;
+                if (in && lr == 0) p.chg[v] = any ? 255 : 128;
             }
         }
         if constexpr (!BF) {

@@ -306,3 +306,19 @@ def test_column_counts_of_one_kernel_and_shared_size_on_one_plan(dag, graph, cal
         D, _, st = dag.sssp_batched(plan, torch.from_numpy(src.view(np.int32)).cuda(), wd, variant, delta)
         assert st["converged"]
         assert np.array_equal(D[:, B - 1].cpu().numpy().view(np.uint32), oracle.dijkstra(g, w, int(src[B - 1])))
+
+
+@pytest.mark.parametrize("B", [5, 20, 36, 130, 261])
+@pytest.mark.parametrize("n", [1, 2, 997])
+def test_runs_sources_anywhere_in_ragged_groups(dag, B, n):
+    # a vertex that is only one column's source, whichever lane and chunk hold the column and wherever the vertex is in
+    # its warp's last, partial group, is read in the first sweep (a cycle: each distance hangs on it)
+    g = I.from_edges(n, np.arange(n) if n > 1 else np.zeros(0, int), (np.arange(n) + 1) % n if n > 1 else np.zeros(0, int))
+    plan = dag.Plan.from_graph(g, "cuda")
+    wd = torch.full((g.m,), 2, dtype=torch.uint8, device="cuda")
+    src = (n - 1 - np.arange(B)) % n
+    for variant in ("sync", "async"):
+        D, _, st = dag.sssp_batched(plan, torch.from_numpy(src.astype(np.int32)).cuda(), wd, variant, 0)
+        assert st["converged"]
+        want = 2 * ((np.arange(n)[:, None] - src[None, :]) % n)
+        assert np.array_equal(D.cpu().numpy().view(np.uint32), want.astype(np.uint32))

@@ -1,0 +1,24 @@
+"""Rules of the kernel sources that no run on one GPU can show."""
+import glob
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2110_01409_gb300", "csrc")
+
+
+def _code(path):
+    with open(path) as f:
+        return re.sub(r"//[^\n]*|/\*.*?\*/", "", f.read(), flags=re.S)
+
+
+def test_no_vote_relies_on_the_lanes_that_happen_to_be_active():
+    # __activemask() does not promise that lanes which diverged have met again. It may pick the lanes that share an
+    # atomic (__match_any_sync: any split of the warp gives the same sums); a vote or a shuffle over it may miss some.
+    seen = 0
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu*"))):
+        for call in re.findall(r"(\w+)\(\s*__activemask\(\)", _code(path)):
+            seen += 1
+            assert call == "__match_any_sync", (os.path.basename(path), call)
+        assert len(re.findall(r"__activemask", _code(path))) == len(re.findall(r"__match_any_sync\(\s*__activemask\(\)",
+                                                                               _code(path)))
+    assert seen
