@@ -501,6 +501,16 @@ int dag_debug_skip_barrier_once(dag_plan* plan, int32_t timeout_ms);
  */
 int dag_debug_stall_staging_once(dag_plan* plan, int32_t timeout_ms);
 
+/*
+ * Test hook for the way out after a wait has given up: the next dag_pagerank,
+ * dag_sssp or dag_pagerank_adjoint (out_plan) solve on this plan starts with
+ * the DAG_ERR_* code recorded on the device, as a CTA whose wait ran out
+ * records it. Every CTA leaves within a sweep, the outputs are not written and
+ * the call returns the code. Resets itself after one solve. code must be
+ * negative.
+ */
+int dag_debug_record_error_once(dag_plan* plan, int32_t code);
+
 #ifdef __cplusplus
 }
 #endif

@@ -189,6 +189,7 @@ struct dag_plan {
     int num_sms = 0;
     long long timeout_ns = dag::DEFAULT_TIMEOUT_NS;
     int skip_barrier_once = 0;
+    int record_error_once = 0;
     int stall_staging_once = 0;
     long long skip_timeout_ns = 0;
     int worker_cap = 0;       // > 0: at most this many CTAs per solve (more rows per CTA)
@@ -263,6 +264,8 @@ size_t sweep_ring_bytes(int mode, int variant);
 // sweep_tma.cu: the asynchronous form's TMA-staged kernel and its ring size.
 const void* sweep_tma_kernel_ptr(int mode, bool frontier);
 size_t sweep_tma_ring_bytes(int mode);
+// Clears the plan's control block for a solve (and sets the error a test asked for).
+int reset_sync(dag_plan* plan, cudaStream_t s);
 // Launches a sweep of nb CTAs: as one cluster when it is small enough (sets p.cluster), else cooperatively.
 int launch_sweep_grid(const void* k, int nb, size_t dyn, SweepParams& p, cudaStream_t s);
 // Smallest shared-memory carveout of kernel k that keeps per_sm CTAs of
@@ -455,7 +458,8 @@ __device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" 
 // returns false. Every thread of the CTA gets the same answer. Relaxed polls,
 // one fence after the last: an acquire per poll emptied the SM's L1 each time.
 // cluster: the grid is one thread-block cluster (a small graph, CLUSTER_MAX), whose hardware barrier orders the CTAs'
-// memory accesses; it waits for the CTAs that have not left, so it needs no limit of its own.
+// memory accesses; it waits for the CTAs that have not left, so it needs no limit of its own. It does not look at the
+// recorded error either: a CTA leaves on that with the sweep's sums (sweep_residual).
 __device__ __forceinline__ bool grid_barrier(SyncBlock* sb, unsigned nblocks, unsigned long long& target,
                                              long long timeout_ns, int cluster = 0)
 {
@@ -499,6 +503,15 @@ static __device__ __noinline__ bool grid_barrier_call(SyncBlock* sb, unsigned nb
                                                       long long timeout_ns, int cluster = 0)
 {
     return grid_barrier(sb, nblocks, target, timeout_ns, cluster);
+}
+
+// The residual of the sweep that used slot `slot`, read behind its barrier, or -1 (a residual is a sum of absolute
+// values or a count) when an error has been recorded: the caller leaves then. A CTA that reads the error a sweep
+// earlier than another does not hold it up: neither barrier waits for one that has left with an error recorded.
+__device__ __forceinline__ double sweep_residual(const SyncBlock* sb, int slot)
+{
+    const double r = ld_relaxed_f64(&sb->acc_res[slot]);
+    return ld_relaxed_i32(&sb->err) != 0 ? -1.0 : r;
 }
 
 template <typename T>

@@ -921,6 +921,13 @@ extern "C" int dag_debug_stall_staging_once(dag_plan* p, int32_t timeout_ms)
     return DAG_OK;
 }
 
+extern "C" int dag_debug_record_error_once(dag_plan* p, int32_t code)
+{
+    if (!p || code >= 0) return set_error(DAG_ERR_INVALID, "bad argument");
+    p->record_error_once = code;
+    return DAG_OK;
+}
+
 extern "C" int dag_debug_skip_barrier_once(dag_plan* p, int32_t timeout_ms)
 {
     if (!p || timeout_ms < 1) return set_error(DAG_ERR_INVALID, "bad argument");

@@ -393,7 +393,7 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_kernel(const SweepParams 
         }
         if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns, p.cluster)) return;
         if (tid == 0) {
-            sh.res = ld_relaxed_f64(&sb->acc_res[slot]);
+            sh.res = sweep_residual(sb, slot);
             sh.gprev = ld_relaxed_f64(&sb->acc_g[slot]);
             if (c == 0) {
                 const int dead = (it + 2) % 3;  // read by everyone before this barrier
@@ -402,6 +402,7 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_kernel(const SweepParams 
             }
         }
         __syncthreads();
+        if (sh.res < 0.0) return;  // an error was recorded
         last_res = sh.res;
         gprev = sh.gprev;
         if (last_res <= tol) {
@@ -481,6 +482,17 @@ int set_l1_carveout(const void* k, int device, int threads, size_t static_smem, 
         DAG_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, pct));
     }
     if (pct_out) *pct_out = pct;
+    return DAG_OK;
+}
+
+int reset_sync(dag_plan* plan, cudaStream_t s)
+{
+    DAG_CUDA(cudaMemsetAsync(plan->sync, 0, sizeof(SyncBlock), s));
+    if (plan->record_error_once) {
+        const int code = plan->record_error_once;
+        plan->record_error_once = 0;
+        DAG_CUDA(cudaMemcpyAsync(&((SyncBlock*)plan->sync)->err, &code, sizeof(int), cudaMemcpyHostToDevice, s));
+    }
     return DAG_OK;
 }
 
@@ -746,7 +758,8 @@ int launch_sweep(dag_plan* plan, int mode, int variant, int delta, SweepParams& 
                           (const void*)p.val, (const void*)p.degf, (const void*)p.x0, (const void*)p.x1})
         if (((uintptr_t)a & 15u) != 0)
             return set_error(DAG_ERR_INVALID, "graph, weight and state arrays must be 16-byte aligned");
-    DAG_CUDA(cudaMemsetAsync(plan->sync, 0, sizeof(SyncBlock), s));
+    rc = reset_sync(plan, s);
+    if (rc) return rc;
     KernelFn k = kernel_for(mode, variant, p.frontier != 0);
     size_t dyn = sweep_ring_bytes(mode, variant) + ((variant == DAG_DELAYED) ? (size_t)cap * 4 : 0);
     DAG_CUDA(cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));

@@ -13,7 +13,8 @@
 // register-staged kernel (sweep_common.cuh). Every wait on a ring mbarrier is
 // bounded by the launch's timeout: when one runs out the CTA records
 // DAG_ERR_BARRIER_TIMEOUT, waits (bounded) for its own copies and leaves, and
-// the other CTAs' grid-barrier waits end on the recorded error.
+// the other CTAs leave on the recorded error: in their grid-barrier wait, or (one
+// cluster) with the sweep's sums.
 //
 // Own block through L1 (DAG_READ_OWN_L1): only the owning CTA writes its
 // vertices, and its barriers order its stores before its later loads, so an
@@ -411,7 +412,7 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_tma_kernel(const SweepPar
                     if (sh.tq[(q + 2) % RING] >= 0)
                         (void)mbar_wait(&sh.fill_bar[(q + 2) % RING], ((q + 2) / RING) & 1u, p.timeout_ns);
                 }
-                return;  // the other CTAs' barrier waits end on the recorded error
+                return;  // the other CTAs leave on the recorded error (grid_barrier, sweep_residual)
             }
             const uint32_t E = row_sums<MODE>(sh);
             const uint32_t E_last = __shfl_sync(0xffffffffu, E, NWARP - 1);
@@ -498,7 +499,7 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_tma_kernel(const SweepPar
         }
         if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns, p.cluster)) return;
         if (tid == 0) {
-            sh.res = ld_relaxed_f64(&sb->acc_res[slot]);
+            sh.res = sweep_residual(sb, slot);
             if (FRONTIER || MODE == MODE_ADJ) sh.gprev = ld_relaxed_f64(&sb->acc_g[slot]);
             if (FRONTIER) sh.cnt[0] = ld_relaxed_i32(&sb->fr_nchg[slot]);
             if (c == 0) {
@@ -511,6 +512,7 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_tma_kernel(const SweepPar
             }
         }
         __syncthreads();
+        if (sh.res < 0.0) return;  // an error was recorded
         last_res = sh.res;
         if (last_res <= tol) {
             converged = true;

@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_kernel(const SweepP
         block_add(sh, res_part, &sb->acc_res[slot], g_part, ((SYNC || MODE == MODE_ADJ) && !BF) ? &sb->acc_g[slot] : nullptr);
         if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns, p.cluster)) return;
         if (tid == 0) {
-            sh.res = ld_relaxed_f64(&sb->acc_res[slot]);
+            sh.res = sweep_residual(sb, slot);
             sh.gprev = ld_relaxed_f64(&sb->acc_g[slot]);
             if (c == 0) {
                 const int dead = (it + 2) % 3;  // read by everyone before this barrier
@@ -279,6 +279,7 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_kernel(const SweepP
             }
         }
         __syncthreads();
+        if (sh.res < 0.0) return;  // an error was recorded
         last_res = sh.res;
         gprev = sh.gprev;
         if (last_res <= tol) {
@@ -543,7 +544,7 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_ordered_kernel(const Swe
         block_add(sh, res_part, &sb->acc_res[slot], g_part, MODE == MODE_ADJ ? &sb->acc_g[slot] : nullptr);
         if (!grid_barrier_call(sb, p.nblocks, bar_target, p.timeout_ns, p.cluster)) return;
         if (tid == 0) {
-            sh.res = ld_relaxed_f64(&sb->acc_res[slot]);
+            sh.res = sweep_residual(sb, slot);
             if (MODE == MODE_ADJ) sh.gprev = ld_relaxed_f64(&sb->acc_g[slot]);
             if (c == 0) {
                 const int dead = (it + 2) % 3;  // read by everyone before this barrier
@@ -552,6 +553,7 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_ordered_kernel(const Swe
             }
         }
         __syncthreads();
+        if (sh.res < 0.0) return;  // an error was recorded
         last_res = sh.res;
         if (last_res <= tol) {
             converged = true;
@@ -763,7 +765,8 @@ int launch_warp_sweep(dag_plan* plan, int mode, int variant, int delta, SweepPar
         p.timeout_ns = plan->skip_timeout_ns;
         plan->skip_barrier_once = 0;
     }
-    DAG_CUDA(cudaMemsetAsync(plan->sync, 0, sizeof(SyncBlock), s));
+    rc = reset_sync(plan, s);
+    if (rc) return rc;
     // stamps of an earlier solve must not pass for this one's
     DAG_CUDA(cudaMemsetAsync(p.wpub, 0,
                              (size_t)(kind == WARP_ORDERED ? part->tiles : part->nblocks) * sizeof(unsigned long long),

@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_frontier_kernel(con
         if (lane == 0 && edges) atomicAdd((unsigned long long*)&sb->edges, (unsigned long long)edges);
         if (!grid_barrier(sb, p.nblocks, bar_target, p.timeout_ns, p.cluster)) return;
         if (tid == 0) {
-            sh.res = ld_relaxed_f64(&sb->acc_res[slot]);
+            sh.res = sweep_residual(sb, slot);
             sh.gprev = ld_relaxed_f64(&sb->acc_g[slot]);
             if (c == 0) {
                 const int dead = (it + 2) % 3;  // read by everyone before this barrier
@@ -372,6 +372,7 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_frontier_kernel(con
             }
         }
         __syncthreads();
+        if (sh.res < 0.0) return;  // an error was recorded
         last_res = sh.res;
         if (last_res <= 0.0) {
             converged = true;

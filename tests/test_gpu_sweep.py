@@ -379,3 +379,31 @@ def test_grids_around_one_cluster(dag, tiles, variant, delta, reads):
     for rd in (reads, "frontier") if reads == "refresh" else (reads,):
         d, st = dag.sssp(plan, 0, _w_dev(w), variant, delta, reads=rd)
         assert st["converged"] and np.array_equal(_u32(d), ref), rd
+
+
+@pytest.mark.parametrize("scale", [10, 16])
+@pytest.mark.parametrize("variant,delta,reads", [("sync", 0, "refresh"), ("async", 0, "refresh"), ("delayed", 64, "refresh"),
+                                                 ("sync", 0, "warp"), ("delayed", 64, "warp"), ("async", 0, "ordered"),
+                                                 ("sync", 0, "frontier"), ("async", 0, "frontier"),
+                                                 ("async", 0, "warp+frontier"), ("async", 0, "ordered+frontier")])
+def test_every_cta_leaves_on_a_recorded_error(dag, scale, variant, delta, reads):
+    # as after a wait that gave up: grids of one cluster (scale 10), whose barrier does not look at the error, and
+    # larger ones leave within a sweep, write nothing and report the code; the plan's next solve is whole
+    g = I.rmat(scale, 16, seed=1)
+    plan = _plan(dag, g)
+    w = I.weights_u32(g, 1)
+    if "frontier" not in reads:
+        out = torch.full((g.n,), -1.0, dtype=torch.float32, device="cuda")
+        plan.debug_record_error_once(dag.ERR_BARRIER_TIMEOUT)
+        with pytest.raises(dag.DagError) as ei:
+            dag.pagerank(plan, 0.85, 1e-6, variant, delta, reads=reads, out=out)
+        assert ei.value.code == dag.ERR_BARRIER_TIMEOUT and bool((out == -1.0).all())
+        r, st = dag.pagerank(plan, 0.85, 1e-6, variant, delta, reads=reads, out=out)
+        assert st["converged"] and abs(float(r.double().sum()) - 1.0) <= 1e-5
+    out = torch.full((g.n,), 7, dtype=torch.int32, device="cuda")
+    plan.debug_record_error_once(dag.ERR_BARRIER_TIMEOUT)
+    with pytest.raises(dag.DagError) as ei:
+        dag.sssp(plan, 0, _w_dev(w), variant, delta, reads=reads, out=out)
+    assert ei.value.code == dag.ERR_BARRIER_TIMEOUT and bool((out == 7).all())
+    d, st = dag.sssp(plan, 0, _w_dev(w), variant, delta, reads=reads, out=out)
+    assert st["converged"] and np.array_equal(_u32(d), oracle.dijkstra(g, w, 0))
