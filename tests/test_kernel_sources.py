@@ -22,3 +22,12 @@ def test_no_vote_relies_on_the_lanes_that_happen_to_be_active():
         assert len(re.findall(r"__activemask", _code(path))) == len(re.findall(r"__match_any_sync\(\s*__activemask\(\)",
                                                                                _code(path)))
     assert seen
+
+
+def test_the_warp_frontiers_marks_cannot_wrap():
+    # a lane's share of a sweep's marks is added to in count_marks only, which stops it at 2^31: with one out-degree below
+    # 2^31 more it still fits 32 bits (a graph that gets there is of the largest size)
+    code = _code(os.path.join(CSRC, "sweep_warp_frontier.cu"))
+    assert re.search(r"unsigned marks = 0u;", code)
+    assert "marks +=" not in code and len(re.findall(r"count_marks\(marks,", code)) == 3
+    assert "marks = min(marks + (unsigned)degree, 1u << 31);" in code and (1 << 31) + (1 << 31) - 1 < 1 << 32
