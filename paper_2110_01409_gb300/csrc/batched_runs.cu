@@ -27,6 +27,7 @@
 // a sweep skips an in-edge whose source changed neither in it nor in the one before (its value is already in the
 // row), and a row with nothing left to read (the conditional updates of Sec. V, at vertex granularity). Distances
 // and the synchronous trajectory are those of the full sweep.
+#include <cfloat>
 #include <climits>
 #include <cstdint>
 
@@ -64,6 +65,21 @@ __device__ __forceinline__ uint32_t comb(uint32_t a, uint32_t b)
 {
     if constexpr (BF) return a < b ? a : b;
     else return __float_as_uint(__uint_as_float(a) + __uint_as_float(b));
+}
+// Adds b to the sum hi + lo, the rounding of hi's addition kept in lo (Knuth's two-sum): FP32 parts on their way to an
+// FP64 sum, without FP64 additions, which issue at two lanes per clock and SM. (An infinite sum has no rounding.)
+__device__ __forceinline__ void two_add(float& hi, float& lo, float b)
+{
+    const float s = hi + b, t = s - hi;
+    if (fabsf(s) <= FLT_MAX) lo += (hi - (s - t)) + (b - t);
+    hi = s;
+}
+// The same with the sum of lane ^ o.
+__device__ __forceinline__ void two_join(float& hi, float& lo, int o)
+{
+    const float b = __shfl_xor_sync(0xffffffffu, hi, o), bl = __shfl_xor_sync(0xffffffffu, lo, o);
+    two_add(hi, lo, b);
+    lo += bl;
 }
 __device__ __forceinline__ uint32_t relax_w(uint32_t du, uint32_t w)
 {
@@ -148,14 +164,14 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
     const bool sync = p.sync != 0;
     const int W = p.nblocks * RUN_WARPS, w = blockIdx.x * RUN_WARPS + warp;
 
-    double* s_T = (double*)smem_raw;                              // [S] teleport totals (PPR)
-    double* s_g = s_T + (BF ? 0 : S);                             // [S] mass on linked vertices, last sweep (PPR)
+    double* s_T = (double*)smem_raw;                              // [S] teleport totals (PPR; async: times g_coef)
+    double* s_g = s_T + (BF ? 0 : S);                             // [S] PPR: mass on linked vertices, last sweep (sync),
+                                                                  // or the CTA's change of the live mass (async)
     float* s_red = (float*)(s_g + (BF ? 0 : S));                  // [RUN_WARPS][S] the warps' per-column sums
     uint32_t* s_head = (uint32_t*)(s_red + RUN_WARPS * S);        // [RUN_WARPS][S] partial of the run's first row
     int* s_last = (int*)(s_head + RUN_WARPS * S);                 // [S] sweeps each column ran
     int* s_run = s_last + S;                                      // [S] 1: the column still runs
-    float* s_live = (float*)(s_run + S);                          // [S] PPR: the CTA's change of the live mass
-    int* s_list = (int*)(s_live + (BF ? 0 : S));                                      // [RUN_WARPS][2][2][32] items: vertex, weight
+    int* s_list = s_run + S;                                      // [RUN_WARPS][2][2][32] items: vertex, weight
     uint32_t* s_ring = (uint32_t*)(s_list + RUN_WARPS * 128);     // [RUN_WARPS][D][SR] fetched rows
     int* list = s_list + warp * 128;
     uint32_t* ring = s_ring + (size_t)warp * D * SR;
@@ -173,6 +189,7 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
     auto from = [&](int q) { return !EVERY || has(q) ? col0(q) : S - 4; };
 
     // per-column sums of the CTA's warps (group 0's lanes hold them), added in a fixed order, one FP64 atomic each
+    // (Bellman-Ford's counts in FP32: only a zero matters, and no sum rounds to it)
     auto cta_sum = [&](const float (&part)[CH][4], double* dst, double* dst2) {
         __syncthreads();
 #pragma unroll
@@ -182,12 +199,16 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
                 for (int e = 0; e < 4; ++e) s_red[warp * S + col0(q) + e] = part[q][e];
         __syncthreads();
         for (int c = tid; c < B; c += NT) {
-            float v = 0.0f;
+            float v = s_red[c], low = 0.0f;
 #pragma unroll
-            for (int k = 0; k < RUN_WARPS; ++k) v += s_red[k * S + c];
-            if (v != 0.0f) {
-                atomicAdd(&dst[c], (double)v);
-                if (dst2) atomicAdd(&dst2[c], (double)v);
+            for (int k = 1; k < RUN_WARPS; ++k) {
+                if constexpr (BF) v += s_red[k * S + c];
+                else two_add(v, low, s_red[k * S + c]);
+            }
+            if (v != 0.0f || low != 0.0f) {
+                const double sum = (double)v + (double)low;
+                atomicAdd(&dst[c], sum);
+                if (dst2) atomicAdd(&dst2[c], sum);
             }
         }
     };
@@ -248,26 +269,33 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
             }
         }
         if constexpr (!BF) {
+            // the groups' FP32 parts, joined in two floats per column
+            float glow[CH][4], tlow[CH][4];
 #pragma unroll
             for (int q = 0; q < CH; ++q)
 #pragma unroll
-                for (int e = 0; e < 4; ++e)
+                for (int e = 0; e < 4; ++e) {
+                    glow[q][e] = tlow[q][e] = 0.0f;
 #pragma unroll
                     for (int o = LPR; o < 32; o <<= 1) {
-                        gpart[q][e] += __shfl_xor_sync(FULL, gpart[q][e], o);
-                        tpart[q][e] += __shfl_xor_sync(FULL, tpart[q][e], o);
+                        two_join(gpart[q][e], glow[q][e], o);
+                        two_join(tpart[q][e], tlow[q][e], o);
                     }
+                }
             cta_sum(tpart, p.T, nullptr);
             cta_sum(gpart, p.acc_g + 2 * B, sync ? nullptr : p.gl);
+            if constexpr (GRP > 1) {
+                cta_sum(tlow, p.T, nullptr);
+                cta_sum(glow, p.acc_g + 2 * B, sync ? nullptr : p.gl);
+            }
         }
     }
     if (!grid_barrier(p.sb, p.nblocks, bar, p.timeout_ns)) return;
     for (int c = tid; c < S; c += NT) {
         if constexpr (!BF) {
-            s_T[c] = c < B ? ld_relaxed_f64(&p.T[c]) : 0.0;
-            s_g[c] = c < B ? ld_relaxed_f64(&p.acc_g[2 * B + c]) : 0.0;
+            s_T[c] = c < B ? (sync ? 1.0 : (double)p.g_coef) * ld_relaxed_f64(&p.T[c]) : 0.0;
+            s_g[c] = sync && c < B ? ld_relaxed_f64(&p.acc_g[2 * B + c]) : 0.0;
         }
-        if (!BF) s_live[c] = 0.0f;
         s_last[c] = 0;
         s_run[c] = c < B ? 1 : 0;
     }
@@ -309,7 +337,7 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
             for (int q = 0; q < CH; ++q)
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    if (mass[q][e] != 0.0f) atomicAdd(&s_live[col0(q) + e], mass[q][e]);
+                    if (mass[q][e] != 0.0f) atomicAdd(&s_g[col0(q) + e], (double)mass[q][e]);
                     mass[q][e] = 0.0f;
                 }
         };
@@ -318,8 +346,8 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
                 give_mass();
                 if ((++turn & (RUN_WARPS - 1)) == 0)
                     for (int c = lane; c < B; c += 32) {
-                        const float v = atomicExch(&s_live[c], 0.0f);
-                        if (v != 0.0f) atomicAdd(&p.gl[c], (double)v);
+                        const double v = __longlong_as_double((long long)atomicExch((unsigned long long*)&s_g[c], 0ULL));
+                        if (v != 0.0) atomicAdd(&p.gl[c], v);
                     }
             }
 #pragma unroll
@@ -328,7 +356,7 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
                 for (int e = 0; e < 4; ++e) {
                     if (!((act[q] >> e) & 1u)) continue;
                     const int c = col0(q) + e;
-                    gt[q][e] = p.g_coef * (float)(s_T[c] - ld_relaxed_f64(&p.gl[c]));  // (FP64 issues slowly here)
+                    gt[q][e] = (float)fma(-(double)p.g_coef, ld_relaxed_f64(&p.gl[c]), s_T[c]);
                 }
         };
         // row v's new values from its sum (every group holds it) and inputs; group 0 stores them
@@ -758,17 +786,15 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
             for (int e = 0; e < 4; ++e) acc[q][e] = ident<BF>();
         }  // runs
         if (ok && pend >= 0) resolve(pend, pend_row);
-        if (!BF && !sync) give_mass();
-
         // ---------------- end of sweep: per-column sums, barrier, stopping rules ----------------
         cta_sum(res, p.acc_res + slot * B, nullptr);
-        if (!BF && !sync)
+        if (!BF) cta_sum(mass, sync ? p.acc_g + slot * B : p.gl, nullptr);
+        if (!BF && !sync)  // what the warps gave during the sweep (cta_sum's barriers stand before and after)
             for (int c = tid; c < B; c += NT) {
-                const float v = s_live[c];  // (cta_sum's barriers stand before and after)
-                if (v != 0.0f) atomicAdd(&p.gl[c], (double)v);
-                s_live[c] = 0.0f;
+                const double v = s_g[c];
+                if (v != 0.0) atomicAdd(&p.gl[c], v);
+                s_g[c] = 0.0;
             }
-        if (!BF && sync) cta_sum(mass, p.acc_g + slot * B, nullptr);
         if (!grid_barrier(p.sb, p.nblocks, bar, p.timeout_ns)) return;
         int still = 0;
         for (int c = tid; c < B; c += NT) {
@@ -854,7 +880,7 @@ size_t run_smem_bytes(bool is_bf, int B)
     const size_t S = (size_t)((B + 3) & ~3);
     const int k = run_shape(B), depth = run_depth(k < 5 ? 1 << k : 32, k > 5 ? 1 << (k - 5) : 1);
     const size_t SR = run_padded(is_bf, k < 5 ? 1 << k : 32, k > 5 ? 1 << (k - 5) : 1) ? (size_t)4 << k : S;
-    return (is_bf ? 0 : 2 * S * 8 + S * 4) + 2 * RUN_WARPS * S * 4 + 2 * S * 4 + RUN_WARPS * 128 * 4 +
+    return (is_bf ? 0 : 2 * S * 8) + 2 * RUN_WARPS * S * 4 + 2 * S * 4 + RUN_WARPS * 128 * 4 +
            (size_t)RUN_WARPS * depth * SR * 4;
 }
 

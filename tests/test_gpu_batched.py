@@ -322,3 +322,23 @@ def test_runs_sources_anywhere_in_ragged_groups(dag, B, n):
         assert st["converged"]
         want = 2 * ((np.arange(n)[:, None] - src[None, :]) % n)
         assert np.array_equal(D.cpu().numpy().view(np.uint32), want.astype(np.uint32))
+
+
+@pytest.mark.parametrize("B", [8, 100, 128])
+@pytest.mark.parametrize("variant", ["sync", "async"])
+def test_runs_dangling_mass_beside_a_large_column_sum(dag, B, variant):
+    # vertex 0 links to itself and holds the column's mass, 1; the seven dangling ones start with half an ulp of it each.
+    # Added up in FP32 over a CTA's warps those vanish from the teleport total, and with them the dangling term, 0.39 of
+    # 0.89 half ulps of their rank. Vertex 0's rank, 1 + 2 x 0.39 half ulps, rounds to 1: the term is d / n of that larger,
+    # 0.05 half ulps.
+    n, d, half = 8, 0.5, 2.0 ** -24
+    V = np.zeros((n, B), dtype=np.float32)
+    V[0, :] = 1.0
+    V[1:, B - 1] = half
+    plan = dag.Plan(torch.tensor([0] + [1] * n, dtype=torch.int32, device="cuda"),
+                    torch.tensor([0], dtype=torch.int32, device="cuda"))
+    R, _, _ = dag.ppr_batched(plan, torch.from_numpy(V).cuda(), d, 1e-12, variant, 0, max_iters=400)
+    dangling = 3.5 * half / (1 - 7 * d / n)
+    want = 0.5 * half + d / n * dangling
+    assert np.abs(R[1:, B - 1].cpu().numpy().astype(np.float64) - want).max() <= 0.06 * half, (R[1, B - 1].item(), want)
+    assert R[0, B - 1].item() == 1.0
