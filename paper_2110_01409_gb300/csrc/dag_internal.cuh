@@ -252,6 +252,8 @@ int sweep_shape(dag_plan* plan, int mode, int variant, int delta, int* nb_out, i
 int settle_shape(dag_plan* plan, int mode, int variant, int delta,
                  const std::function<int(int nblocks, int* max_rows)>& partition, int* nb_out, int* cap_out,
                  int* clamped_out, Shape* how = nullptr);
+// A row's weight beside its in-edges in the cuts of nb CTAs' blocks, tiles of at most cap rows (0: no cap).
+int cta_row_weight(const dag_plan* plan, int mode, int variant, int cap, int nb);
 // Rows a tile of a delayed sweep may complete (0: no cap): a buffer of delta
 // rows can only be flushed at a tile end.
 inline int delayed_row_cap(int variant, int delta) { return (variant == DAG_DELAYED && delta > 0 && delta < TILE) ? delta : 0; }

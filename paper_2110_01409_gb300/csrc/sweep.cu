@@ -665,7 +665,7 @@ int settle_shape(dag_plan* plan, int mode, int variant, int delta,
 // 12.05, 12.89 (0.5 M vertices 1.61, 1.67, 1.51, 2.08), delta 256 4.93, 4.84, 5.06, 5.35.
 // A grid of a CTA or more per tile takes k, so that blocks are the tiles it was sized for (Bellman-Ford, 1,000 vertices,
 // delta 32: 113 us a call, 129 with two tiles in some blocks).
-static int cta_row_weight(const dag_plan* plan, int mode, int variant, int cap, int nb)
+int cta_row_weight(const dag_plan* plan, int mode, int variant, int cap, int nb)
 {
     const bool bf = mode == MODE_BF || mode == MODE_BF8;
     const int k = tile_row_weight(cap);

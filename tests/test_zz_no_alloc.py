@@ -104,3 +104,14 @@ def test_noalloc_rejects_colidx_out_of_range(dag):
     r, st = dag.pagerank_noalloc(rowptr, colidx, 0.85, 1e-6, "delayed", 16)
     assert st["converged"]
     assert _l1(r.cpu(), torch.from_numpy(oracle.dense_pagerank(g, 0.85))) <= 1e-5
+
+
+@pytest.mark.parametrize("variant,delta", [("sync", 0), ("async", 0), ("delayed", 1), ("delayed", 256)])
+def test_noalloc_largest_graph(dag, variant, delta):
+    # the most vertices there may be, half of them without in-edges: blocks cut by the rows' weight, their tiles all in
+    # the scratch array
+    g = I.rmat(20, 15, seed=4)
+    rowptr, colidx = _dev(g)
+    ref, _ = dag.pagerank(dag.Plan(rowptr, colidx), 0.85, 1e-6, "sync", 0)
+    r, st = dag.pagerank_noalloc(rowptr, colidx, 0.85, 1e-6, variant, delta)
+    assert st["converged"] and _l1(r, ref) <= 2e-5  # each within d / (1 - d) tol = 5.7e-6 of the fixed point
