@@ -408,7 +408,7 @@ def gathers_coherent(variant, delta, reads):
 
 
 SWEEP_SOURCES = ("sweep.cu", "sweep_tma.cu", "sweep_warp.cu", "sweep_warp_frontier.cu", "sweep_warp.cuh",
-                 "sweep_common.cuh", "dag_internal.cuh")
+                 "sweep_edges.cuh", "sweep_common.cuh", "dag_internal.cuh")
 
 
 def sweep_source_hash():

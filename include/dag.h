@@ -16,9 +16,11 @@
  *  - Graphs are in-edge CSR: colidx[rowptr[v] .. rowptr[v+1]) are the sources u
  *    of the edges u -> v. rowptr/colidx are int32 (m < 2^31).
  *  - rowptr, colidx and the per-edge weight / value arrays start on a 16-byte
- *    boundary (any cudaMalloc or fresh torch allocation does); the sweeps copy
- *    them with TMA bulk copies. A solve given a misaligned array returns
- *    DAG_ERR_INVALID.
+ *    boundary (any cudaMalloc or fresh torch allocation does); the sweeps over
+ *    CTA tiles copy them with TMA bulk copies, which may read on to the end of
+ *    an array's last 16 bytes. A solve on CTA tiles given a misaligned array
+ *    returns DAG_ERR_INVALID; the warp-worker and the batched solves take
+ *    arrays aligned to their elements, and read nothing outside them.
  *  - Pointers named d_* are DEVICE pointers on the current CUDA device; h_*
  *    are HOST pointers. All arrays belong to the caller; the library keeps no
  *    pointer to them after the call returns, except that a plan keeps the CSR

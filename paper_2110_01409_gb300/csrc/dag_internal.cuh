@@ -86,6 +86,7 @@ constexpr size_t SYNC_HEAD = offsetof(SyncBlock, stripe);
 // Parameters of one sweep launch.
 struct SweepParams {
     int n;
+    int m;                  // in-edges of the whole graph (warp sweeps)
     int nblocks;
     const int* rowptr;
     const int* colidx;

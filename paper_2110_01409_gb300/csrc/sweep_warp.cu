@@ -756,6 +756,7 @@ int launch_warp_sweep(dag_plan* plan, int mode, int variant, int delta, SweepPar
     p.tile_nz = part->tile_nz;
     p.wpub = kind == WARP_ORDERED ? part->tpub : part->wpub;
     p.ntiles = part->tiles;
+    p.m = (int)plan->m;
     p.sync = plan->sync;
     p.timeout_ns = plan->timeout_ns;
     p.skip_barrier_cta0 = 0;
@@ -808,6 +809,7 @@ int sweep_rows(dag_plan* plan, int mode, int lo, int hi, SweepParams& p, double*
     int rc = get_warp_partition_range(plan, nb * WWARPS, WTILE, warp_row_weight(WARP_RUNS, mode), lo, hi, &part, s);
     if (rc) return rc;
     p.nblocks = nb;
+    p.m = (int)plan->m;
     p.max_iters = 1;
     p.tol = 0.0;
     p.delta = 0;

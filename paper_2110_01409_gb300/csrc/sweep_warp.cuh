@@ -9,6 +9,7 @@
 #include <cstdint>
 
 #include "sweep_common.cuh"
+#include "sweep_edges.cuh"
 
 namespace dag {
 
@@ -63,16 +64,28 @@ __device__ __forceinline__ void wcp16(void* dst, uintptr_t src, uint64_t pol)
                  ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "l"(pol) : "memory");
 }
 
+__device__ __forceinline__ void wcp4(void* dst, const int* src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;"
+                 ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+
 // Starts the copies of tile c's edge sources into the warp's buffer: whole 16-byte granules around the wanted
-// elements, whatever the array's alignment.
+// elements, whatever the array's alignment, or at the array's ends the wanted elements (sweep_edges.cuh).
 template <int MODE, int WIPT>
 __device__ __forceinline__ void wissue_col(WarpShared<MODE, WIPT>& sh, const SweepParams& p, const WCoord& c, int wl, int lane,
                                            uint64_t pol_edge)
 {
     if (c.b1 <= c.b0) return;
-    const uintptr_t a = (uintptr_t)(p.colidx + c.b0);
-    const int n = ((int)(a & 15u) + 4 * (c.b1 - c.b0) + 15) >> 4;
-    for (int k = lane; k < n; k += 32) wcp16((char*)sh.col[wl] + 16 * k, (a & ~(uintptr_t)15) + 16 * k, pol_edge);
+    const int mis = (int)((uintptr_t)p.colidx >> 2) & 3, n = edge_granules(mis, c.b0, c.b1);
+    const int lead = edge_lead(mis, c.b0);
+    if (edge_granules_inside(mis, c.b0, c.b1, p.m)) {
+        const uintptr_t a = (uintptr_t)(p.colidx + c.b0 - lead);
+        for (int k = lane; k < n; k += 32) wcp16((char*)sh.col[wl] + 16 * k, a + 16 * k, pol_edge);
+    } else {
+#pragma unroll 1
+        for (int j = lane; j < c.b1 - c.b0; j += 32) wcp4(sh.col[wl] + lead + j, p.colidx + c.b0 + j);
+    }
 }
 __device__ __forceinline__ void wcommit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 // The warp's copies have landed, and every lane is done with what it read before.
@@ -109,7 +122,7 @@ __device__ __forceinline__ void wgather(WStage<MODE, WIPT>& st, WarpShared<MODE,
     st.NB = c.b1 - c.b0;
     st.rp0 = (int)ld_vertex_b32(p.rowptr + st.a0, pol_vertex);
     st.re0 = lane < st.NA ? (int)ld_vertex_b32(p.rowptr + st.a0 + lane + 1, pol_vertex) : 0;
-    const int* col = sh.col[wl] + (((uintptr_t)(p.colidx + c.b0) >> 2) & 3u);
+    const int* col = sh.col[wl] + edge_lead((int)((uintptr_t)p.colidx >> 2) & 3, c.b0);
     uint32_t aux[MODE == MODE_PR ? 1 : WIPT];
 #pragma unroll
     for (int q = 0; q < WIPT; ++q) {

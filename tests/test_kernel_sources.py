@@ -1,7 +1,9 @@
 """Rules of the kernel sources that no run on one GPU can show."""
+import ctypes
 import glob
 import os
 import re
+import subprocess
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2110_01409_gb300", "csrc")
 
@@ -31,3 +33,43 @@ def test_the_warp_frontiers_marks_cannot_wrap():
     assert re.search(r"unsigned marks = 0u;", code)
     assert "marks +=" not in code and len(re.findall(r"count_marks\(marks,", code)) == 3
     assert "marks = min(marks + (unsigned)degree, 1u << 31);" in code and (1 << 31) + (1 << 31) - 1 < 1 << 32
+
+
+def test_edge_copies_stay_inside_the_array(tmp_path):
+    # a warp tile's copy of its edge sources, for arrays at every offset to a 16-byte boundary and every cut of them: the
+    # elements read lie in the array and the wanted ones land where the gathers look for them
+    src = tmp_path / "edges.cpp"
+    src.write_text('''
+#include "sweep_edges.cuh"
+#include <algorithm>
+// 0, or the first tile that reads outside [0, m) or misses an element, as 1 + ((mis * 64 + m) * 64 + b0) * 64 + b1
+extern "C" int check() {
+    for (int mis = 0; mis < 4; ++mis)
+        for (int m = 1; m < 40; ++m)
+            for (int b0 = 0; b0 < m; ++b0)
+                for (int b1 = b0 + 1; b1 <= m; ++b1) {
+                    int col[64];
+                    std::fill(col, col + 64, -1);
+                    bool ok = true;
+                    auto copy = [&](int at, int e) { ok = ok && e >= 0 && e < m; col[at] = e; };
+                    const int n = dag::edge_granules(mis, b0, b1), lead = dag::edge_lead(mis, b0);
+                    ok = ok && ((b0 - lead + mis) & 3) == 0;  // the granules start on a 16-byte boundary
+                    if (dag::edge_granules_inside(mis, b0, b1, m))
+                        for (int i = 0; i < 4 * n; ++i) copy(i, b0 - lead + i);
+                    else {
+                        ok = ok && (b0 < 4 || b1 > m - 4);
+                        for (int j = 0; j < b1 - b0; ++j) copy(lead + j, b0 + j);
+                    }
+                    for (int e = b0; e < b1; ++e) ok = ok && col[lead + e - b0] == e;
+                    if (!ok || 4 * n > (b1 - b0) + 8) return 1 + ((mis * 64 + m) * 64 + b0) * 64 + b1;
+                }
+    return 0;
+}
+''')
+    lib = tmp_path / "edges.so"
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-x", "c++", "-I", CSRC, str(src), "-o", str(lib)],
+                   check=True)
+    assert ctypes.CDLL(str(lib)).check() == 0
+    # and the kernels use this arithmetic
+    code = _code(os.path.join(CSRC, "sweep_warp.cuh"))
+    assert "if (edge_granules_inside(mis, c.b0, c.b1, p.m)) {" in code and code.count("wcp16(") == 2
