@@ -513,6 +513,13 @@ int dag_debug_stall_staging_once(dag_plan* plan, int32_t timeout_ms);
  */
 int dag_debug_record_error_once(dag_plan* plan, int32_t code);
 
+/*
+ * Test hook for batched solves on a full device: scratch of the merge-path
+ * runs (dag_plan_set_batched_wide) above `bytes` counts as not fitting, as an
+ * allocation that fails, and such solves run on the kernel that needs none.
+ */
+int dag_debug_limit_batched_scratch(dag_plan* plan, int64_t bytes);
+
 #ifdef __cplusplus
 }
 #endif

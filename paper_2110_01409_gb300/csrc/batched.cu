@@ -585,7 +585,7 @@ static int launch_on(bool runs, dag_plan* plan, int is_bf, int variant, int delt
         dev_free(plan->bruns);
         plan->bruns = nullptr;
         plan->bruns_bytes = 0;
-        if (dev_alloc(&plan->bruns, rbytes) != cudaSuccess) {
+        if (rbytes > plan->bruns_limit || dev_alloc(&plan->bruns, rbytes) != cudaSuccess) {
             cudaGetLastError();
             return set_error(DAG_ERR_NOMEM, "batched workspace allocation failed");
         }
@@ -671,7 +671,8 @@ static int launch_on(bool runs, dag_plan* plan, int is_bf, int variant, int delt
 }
 
 // Runs of the merge path but for the delayed form; where their scratch (partials, a padded copy of rows that are not
-// whole 16-byte chunks) does not fit on the device, the 32-column kernel, whose in-place forms take none.
+// whole 16-byte chunks) does not fit on the device, the 32-column kernel, whose in-place forms take none: what the
+// attempt allocated is given back first.
 int launch_batched(dag_plan* plan, int is_bf, int variant, int delta, int max_iters, int B, float d, double tol,
                    const void* V_or_src, const uint32_t* w, void* out, int* iters, dag_batch_stats* st,
                    cudaStream_t s)
@@ -680,10 +681,26 @@ int launch_batched(dag_plan* plan, int is_bf, int variant, int delta, int max_it
     const int rc = launch_on(runs, plan, is_bf, variant, delta, max_iters, B, d, tol, V_or_src, w, out, iters, st, s);
     if (!runs || rc != DAG_ERR_NOMEM) return rc;
     cudaGetLastError();  // the allocation's
+    DAG_CUDA(cudaFree(plan->bx));  // (waits for the device; the kernel's second iterate is allocated afresh)
+    plan->bx = nullptr;
+    plan->bx_bytes = 0;
     return launch_on(false, plan, is_bf, variant, delta, max_iters, B, d, tol, V_or_src, w, out, iters, st, s);
 }
 
 }  // namespace dag
+
+extern "C" int dag_debug_limit_batched_scratch(dag_plan* plan, int64_t bytes)
+{
+    if (!plan || bytes < 0) return dag::set_error(DAG_ERR_INVALID, "bad argument");
+    if ((unsigned long long)bytes < plan->bruns_bytes) {
+        DAG_CUDA(cudaDeviceSynchronize());  // a solve in flight may still use it
+        dag::dev_free(plan->bruns);
+        plan->bruns = nullptr;
+        plan->bruns_bytes = 0;
+    }
+    plan->bruns_limit = (size_t)bytes;
+    return DAG_OK;
+}
 
 extern "C" int dag_plan_set_batched_wide(dag_plan* plan, int32_t on)
 {

@@ -223,6 +223,7 @@ struct dag_plan {
     size_t bsync_bytes = 0;
     void* bruns = nullptr;      // runs: published partials and (Bellman-Ford) the vertices' last changes
     size_t bruns_bytes = 0;
+    size_t bruns_limit = SIZE_MAX;  // test hook: more than this does not fit
 };
 
 namespace dag {

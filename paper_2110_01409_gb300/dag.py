@@ -41,7 +41,7 @@ EXPORTS = (
     "dag_pagerank", "dag_sssp", "dag_ppr_batched", "dag_sssp_batched", "dag_transpose",
     "dag_normalize_weights", "dag_pagerank_adjoint", "dag_strerror", "dag_last_error_message",
     "dag_debug_skip_barrier_once", "dag_debug_stall_staging_once",
-    "dag_debug_record_error_once", "dag_tile_items", "dag_pagerank_noalloc", "dag_gather_f32", "dag_plan_set_worker_cap",
+    "dag_debug_record_error_once", "dag_debug_limit_batched_scratch", "dag_tile_items", "dag_pagerank_noalloc", "dag_gather_f32", "dag_plan_set_worker_cap",
     "dag_sssp_u8", "dag_probe_gather", "dag_access_matrix", "dag_plan_set_batched_graph", "dag_warp_tile_items",
     "dag_plan_set_warp_tile", "dag_plan_last_status", "dag_sssp_batched_u8", "dag_rank_to_state",
     "dag_state_to_rank", "dag_pagerank_sweep_rows", "dag_sssp_sweep_rows", "dag_plan_set_warp_frontier_marks",
@@ -113,6 +113,7 @@ def lib():
             L.dag_debug_skip_barrier_once.argtypes = [_vp, _i32]
             L.dag_debug_stall_staging_once.argtypes = [_vp, _i32]
             L.dag_debug_record_error_once.argtypes = [_vp, _i32]
+            L.dag_debug_limit_batched_scratch.argtypes = [_vp, ctypes.c_int64]
             L.dag_tile_items.restype = _i32
             L.dag_warp_tile_items.restype = _i32
             L.dag_warp_tile_items.argtypes = [_vp]
@@ -259,6 +260,9 @@ class Plan:
 
     def debug_record_error_once(self, code: int):
         _raise(lib().dag_debug_record_error_once(self.h, code), False)
+
+    def debug_limit_batched_scratch(self, nbytes: int):
+        _raise(lib().dag_debug_limit_batched_scratch(self.h, nbytes), False)
 
 
 def pagerank(plan: Plan, d=0.85, tol=1e-6, variant="delayed", delta=256, max_iters=1000, teleport=None,

@@ -93,6 +93,7 @@ def test_null_arguments_are_refused_without_a_gpu(lib):
         "dag_debug_skip_barrier_once": lambda: lib.dag_debug_skip_barrier_once(N, 100),
         "dag_debug_stall_staging_once": lambda: lib.dag_debug_stall_staging_once(N, 100),
         "dag_debug_record_error_once": lambda: lib.dag_debug_record_error_once(N, -3),
+        "dag_debug_limit_batched_scratch": lambda: lib.dag_debug_limit_batched_scratch(N, 0),
     }
     for name, call in calls.items():
         assert call() == -1, name

@@ -342,3 +342,31 @@ def test_runs_dangling_mass_beside_a_large_column_sum(dag, B, variant):
     want = 0.5 * half + d / n * dangling
     assert np.abs(R[1:, B - 1].cpu().numpy().astype(np.float64) - want).max() <= 0.06 * half, (R[1, B - 1].item(), want)
     assert R[0, B - 1].item() == 1.0
+
+
+@pytest.mark.parametrize("variant", ["sync", "async"])
+def test_runs_whose_scratch_does_not_fit(dag, variant):
+    # the solve runs on the 32-column kernel, with the same results, and the plan keeps nothing of the attempt: no padded
+    # copy of the state (30 columns, rows of 32: 240 MB) beside the synchronous form's second buffer
+    g = I.rmat(21, 2, seed=3)
+    B = 30
+    plan = dag.Plan.from_graph(g, "cuda")
+    V = torch.zeros((g.n, B), device="cuda")
+    src = I.sources(g, B, seed=1)
+    V[torch.from_numpy(src.astype(np.int64)).cuda(), torch.arange(B, device="cuda")] = 1.0
+    out = torch.empty_like(V)
+    plan.set_batched_wide(False)
+    ref, it0, _ = dag.ppr_batched(plan, V, 0.85, 1e-6, variant, 0)
+    plan.set_batched_wide(True)
+    plan.debug_limit_batched_scratch(0)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    _, it1, st = dag.ppr_batched(plan, V, 0.85, 1e-6, variant, 0, out=out)
+    assert before - torch.cuda.mem_get_info()[0] < 32 << 20
+    assert st["converged"]
+    if variant == "sync":
+        assert torch.equal(it0, it1)
+    assert float((out - ref).abs().sum(0).max()) <= 2e-5
+    plan.debug_limit_batched_scratch(1 << 40)
+    R, _, st = dag.ppr_batched(plan, V, 0.85, 1e-6, variant, 0)
+    assert st["converged"] and float((R - ref).abs().sum(0).max()) <= 2e-5
