@@ -266,6 +266,40 @@ def test_runs_any_column_count(dag, B, variant):
                 assert its[c] == oracle.sssp(g, w, int(srcs[c]), oracle.SYNC)[1]
 
 
+@pytest.mark.parametrize("cap", [1, 2])
+@pytest.mark.parametrize("B", [1, 3, 6, 12, 20, 33, 72, 130, 300, 1024])
+@pytest.mark.parametrize("variant", ["sync", "async"])
+def test_several_runs_a_warp(dag, B, variant, cap):
+    # one or two CTAs: each warp takes 2 to 15 runs (the graph's weight by a run's 1,024, or 256 above 128 columns;
+    # Bellman-Ford of up to 128 columns on two CTAs one), carries the row it began inside a run from one run to the next,
+    # and looks back over runs of its own and of other warps
+    g = _hub_graph()
+    plan = dag.Plan.from_graph(g, "cuda")
+    plan.set_worker_cap(cap)
+    V = I.teleport_matrix(g.n, I.ppr_seed_sets(g.n, B, seed=4))
+    w = I.weights_u32(g, 9) & 0xFF
+    srcs = np.resize(I.sources(g, min(B, 300), seed=6), B)
+    cols = sorted({0, B // 2, B - 1})
+    R, iters, st = dag.ppr_batched(plan, torch.from_numpy(V).cuda(), 0.85, 1e-5, variant, 0)
+    assert st["converged"] and st["workers"] == cap and st["column_sweeps"] == int(iters.sum())
+    Rn = R.cpu().numpy().astype(np.float64)
+    for c in cols:
+        rstar = oracle.pagerank_fixed_point(g, 0.85, tele=V[:, c].astype(np.float64), tol=1e-12)
+        # d / (1 - d) tol of L1 error, and an eighth for the FP32 parts of the sums: with so few workers a lane adds 375
+        # rows' ranks, two hubs of a seventh among them, and a synchronous sweep's residual stays at up to 7e-6
+        # (the 32-column kernel's at 6e-5)
+        assert np.abs(Rn[:, c] - rstar).sum() <= 5.7e-5 * 1.125, c
+    sd = torch.from_numpy(srcs.view(np.int32)).cuda()
+    for wd in (torch.from_numpy(w.astype(np.uint8)).cuda(), torch.from_numpy(w.view(np.int32)).cuda()):
+        D, iters, st = dag.sssp_batched(plan, sd, wd, variant, 0)
+        assert st["converged"]
+        Dn, its = D.cpu().numpy().view(np.uint32), iters.cpu().numpy()
+        for c in cols:
+            assert np.array_equal(Dn[:, c], oracle.dijkstra(g, w, int(srcs[c]))), c
+            if variant == "sync":
+                assert its[c] == oracle.sssp(g, w, int(srcs[c]), oracle.SYNC)[1]
+
+
 @pytest.mark.parametrize("variant", ["sync", "async"])
 def test_runs_long_path_and_sweep_limit(dag, variant):
     # 600 sweeps: the last-change byte wraps twice; a solve stopped early reports its sweeps

@@ -357,28 +357,34 @@ def test_last_status_copied_on_the_device(dag):
 
 
 @pytest.mark.parametrize("tiles", [1, 2, 8, 9, 16, 17])
-@pytest.mark.parametrize("variant,delta,reads", [("sync", 0, "refresh"), ("async", 0, "refresh"),
+@pytest.mark.parametrize("variant,delta,reads", [("sync", 0, "refresh"), ("async", 0, "refresh"), ("delayed", 64, "refresh"),
                                                  ("async", 0, "ordered"), ("sync", 0, "warp")])
 def test_grids_around_one_cluster(dag, tiles, variant, delta, reads):
     # exactly `tiles` CTA tiles (or as many CTAs of warps): one cluster up to 16 CTAs (8 is the portable size),
-    # the memory barrier above
-    per = 1792 if reads == "refresh" else 8 * 32 * 5
-    n = 12 * tiles + 60  # so many vertices that so many distinct edges exist
-    m = tiles * per - n
+    # the memory barrier above. A tile of at most 64 rows takes 1,792 / 64 = 28 items of each.
+    warp = reads != "refresh"
+    per, row = (8 * 32 * 5 if warp else 1792), (28 if delta else 1)
+    n = 40 * tiles if delta else 12 * tiles + 60  # so many vertices that so many distinct edges exist
+    m = tiles * per - row * n
     rng = np.random.default_rng(tiles)
     k = rng.permutation(n * (n - 1))[:m]
     s, t = k // (n - 1), k % (n - 1)
     g = _from_edges(n, s, t + (t >= s))
     assert g.m == m
     plan = _plan(dag, g)
+    plan.set_warp_tile(5)
+    grid = max(2, tiles) * (8 if warp else 1)  # warp forms count their warps
     rstar = oracle.dense_pagerank(g, 0.85)
     r, st = dag.pagerank(plan, 0.85, 1e-6, variant, delta, reads=reads)
     assert st["converged"] and _l1(r, rstar) <= 1e-5, st
+    assert st["workers"] == grid
     w = I.weights_u32(g, 1)
     ref = oracle.dijkstra(g, w, 0)
-    for rd in (reads, "frontier") if reads == "refresh" else (reads,):
+    with_frontier = {"refresh": "frontier", "ordered": "ordered+frontier", "warp": None}[reads]
+    for rd in (reads, with_frontier) if with_frontier and not delta else (reads,):
         d, st = dag.sssp(plan, 0, _w_dev(w), variant, delta, reads=rd)
         assert st["converged"] and np.array_equal(_u32(d), ref), rd
+        assert st["workers"] == grid, rd
 
 
 @pytest.mark.parametrize("scale", [10, 16])
