@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_kernel(const SweepParams 
             }
         }
         __syncthreads();
-        if (sh.res < 0.0) return;  // an error was recorded
+        if (sweep_failed(sh.res)) return;  // an error was recorded
         last_res = sh.res;
         gprev = sh.gprev;
         if (last_res <= tol) {

@@ -512,7 +512,7 @@ __global__ void __launch_bounds__(NT, MINBLOCKS) sweep_tma_kernel(const SweepPar
             }
         }
         __syncthreads();
-        if (sh.res < 0.0) return;  // an error was recorded
+        if (sweep_failed(sh.res)) return;  // an error was recorded
         last_res = sh.res;
         if (last_res <= tol) {
             converged = true;

@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_kernel(const SweepP
             }
         }
         __syncthreads();
-        if (sh.res < 0.0) return;  // an error was recorded
+        if (sweep_failed(sh.res)) return;  // an error was recorded
         last_res = sh.res;
         gprev = sh.gprev;
         if (last_res <= tol) {
@@ -553,7 +553,7 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_ordered_kernel(const Swe
             }
         }
         __syncthreads();
-        if (sh.res < 0.0) return;  // an error was recorded
+        if (sweep_failed(sh.res)) return;  // an error was recorded
         last_res = sh.res;
         if (last_res <= tol) {
             converged = true;

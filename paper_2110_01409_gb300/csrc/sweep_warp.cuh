@@ -77,11 +77,10 @@ __device__ __forceinline__ void wissue_col(WarpShared<MODE, WIPT>& sh, const Swe
                                            uint64_t pol_edge)
 {
     if (c.b1 <= c.b0) return;
-    const int mis = (int)((uintptr_t)p.colidx >> 2) & 3, n = edge_granules(mis, c.b0, c.b1);
-    const int lead = edge_lead(mis, c.b0);
-    if (edge_granules_inside(mis, c.b0, c.b1, p.m)) {
-        const uintptr_t a = (uintptr_t)(p.colidx + c.b0 - lead);
-        for (int k = lane; k < n; k += 32) wcp16((char*)sh.col[wl] + 16 * k, a + 16 * k, pol_edge);
+    const uintptr_t at = (uintptr_t)(p.colidx + c.b0);
+    const int lead = edge_lead(at), n = edge_granules(lead, c.b1 - c.b0);
+    if (edge_granules_inside(lead, c.b0, c.b1, p.m)) {
+        for (int k = lane; k < n; k += 32) wcp16((char*)sh.col[wl] + 16 * k, (at & ~(uintptr_t)15) + 16 * k, pol_edge);
     } else {
 #pragma unroll 1
         for (int j = lane; j < c.b1 - c.b0; j += 32) wcp4(sh.col[wl] + lead + j, p.colidx + c.b0 + j);
@@ -122,7 +121,7 @@ __device__ __forceinline__ void wgather(WStage<MODE, WIPT>& st, WarpShared<MODE,
     st.NB = c.b1 - c.b0;
     st.rp0 = (int)ld_vertex_b32(p.rowptr + st.a0, pol_vertex);
     st.re0 = lane < st.NA ? (int)ld_vertex_b32(p.rowptr + st.a0 + lane + 1, pol_vertex) : 0;
-    const int* col = sh.col[wl] + edge_lead((int)((uintptr_t)p.colidx >> 2) & 3, c.b0);
+    const int* col = sh.col[wl] + edge_lead((uintptr_t)(p.colidx + c.b0));
     uint32_t aux[MODE == MODE_PR ? 1 : WIPT];
 #pragma unroll
     for (int q = 0; q < WIPT; ++q) {

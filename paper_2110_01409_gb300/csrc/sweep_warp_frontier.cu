@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(NT, WMINBLOCKS) sweep_warp_frontier_kernel(con
             }
         }
         __syncthreads();
-        if (sh.res < 0.0) return;  // an error was recorded
+        if (sweep_failed(sh.res)) return;  // an error was recorded
         last_res = sh.res;
         if (last_res <= 0.0) {
             converged = true;

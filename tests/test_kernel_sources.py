@@ -52,12 +52,12 @@ extern "C" int check() {
                     std::fill(col, col + 64, -1);
                     bool ok = true;
                     auto copy = [&](int at, int e) { ok = ok && e >= 0 && e < m; col[at] = e; };
-                    const int n = dag::edge_granules(mis, b0, b1), lead = dag::edge_lead(mis, b0);
+                    const int lead = dag::edge_lead(4096 + 4 * (mis + b0)), n = dag::edge_granules(lead, b1 - b0);
                     ok = ok && ((b0 - lead + mis) & 3) == 0;  // the granules start on a 16-byte boundary
-                    if (dag::edge_granules_inside(mis, b0, b1, m))
+                    if (dag::edge_granules_inside(lead, b0, b1, m))
                         for (int i = 0; i < 4 * n; ++i) copy(i, b0 - lead + i);
                     else {
-                        ok = ok && (b0 < 4 || b1 > m - 4);
+                        ok = ok && (b0 < 3 || b1 > m - 3);
                         for (int j = 0; j < b1 - b0; ++j) copy(lead + j, b0 + j);
                     }
                     for (int e = b0; e < b1; ++e) ok = ok && col[lead + e - b0] == e;
@@ -72,4 +72,4 @@ extern "C" int check() {
     assert ctypes.CDLL(str(lib)).check() == 0
     # and the kernels use this arithmetic
     code = _code(os.path.join(CSRC, "sweep_warp.cuh"))
-    assert "if (edge_granules_inside(mis, c.b0, c.b1, p.m)) {" in code and code.count("wcp16(") == 2
+    assert "if (edge_granules_inside(lead, c.b0, c.b1, p.m)) {" in code and code.count("wcp16(") == 2
