@@ -20,8 +20,8 @@
 //
 // Measured (RMAT, against a CTA block of whole rows walked in tiles by eight warps with a barrier per tile, and a
 // warp of 32 columns for other column counts): PPR of 256 columns at 1 M vertices 66.5 -> 26.3 ms, of 20 columns at
-// 100 K vertices 7.06 -> 1.05 ms (a hub's row was one warp's), Bellman-Ford of 64 columns at 1 M vertices 24.4 -> 7.5.
-// Slower than that kernel on small uniform graphs of 32 columns only (3 K vertices, PPR: 165 -> 200 us).
+// 100 K vertices 7.06 -> 1.05 ms (a hub's row was one warp's), Bellman-Ford of 64 columns at 1 M vertices 24.4 -> 7.5;
+// small uniform graphs the least: PPR of 32 columns at 3 K vertices 163 -> 146 us.
 //
 // Bellman-Ford reads only what can lower something: chg[u] is the last sweep that lowered any of u's columns, and
 // a sweep skips an in-edge whose source changed neither in it nor in the one before (its value is already in the
@@ -165,13 +165,13 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
     const int W = p.nblocks * RUN_WARPS, w = blockIdx.x * RUN_WARPS + warp;
 
     double* s_T = (double*)smem_raw;                              // [S] teleport totals (PPR; async: times g_coef)
-    double* s_g = s_T + (BF ? 0 : S);                             // [S] PPR: mass on linked vertices, last sweep (sync),
-                                                                  // or the CTA's change of the live mass (async)
-    float* s_red = (float*)(s_g + (BF ? 0 : S));                  // [RUN_WARPS][S] the warps' per-column sums
+    double* s_live = s_T + (BF ? 0 : S);                          // [S] the CTA's change of the live mass (async PPR)
+    float* s_red = (float*)(s_live + (BF ? 0 : S));               // [RUN_WARPS][S] the warps' per-column sums
     uint32_t* s_head = (uint32_t*)(s_red + RUN_WARPS * S);        // [RUN_WARPS][S] partial of the run's first row
     int* s_last = (int*)(s_head + RUN_WARPS * S);                 // [S] sweeps each column ran
     int* s_run = s_last + S;                                      // [S] 1: the column still runs
-    int* s_list = s_run + S;                                      // [RUN_WARPS][2][2][32] items: vertex, weight
+    float* s_gt = (float*)(s_run + S);                            // [S] the dangling term at the start of a sweep (PPR)
+    int* s_list = (int*)(s_gt + (BF ? 0 : S));                    // [RUN_WARPS][2][2][32] items: vertex, weight
     uint32_t* s_ring = (uint32_t*)(s_list + RUN_WARPS * 128);     // [RUN_WARPS][D][SR] fetched rows
     int* list = s_list + warp * 128;
     uint32_t* ring = s_ring + (size_t)warp * D * SR;
@@ -187,6 +187,11 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
     auto has = [&](int q) { return WHOLE || lr + 32 * q < NCH; };
     // EVERY: a lane without columns copies the row's last four too (and never stores them), which saves the branch
     auto from = [&](int q) { return !EVERY || has(q) ? col0(q) : S - 4; };
+
+    // a column's dangling term from its mass on linked vertices (FP64 issues slowly here: once per column where it can be)
+    auto dangling = [&](double linked, double T) {
+        return sync ? (float)((double)p.g_coef * (T - linked)) : (float)fma(-(double)p.g_coef, linked, T);
+    };
 
     // per-column sums of the CTA's warps (group 0's lanes hold them), added in a fixed order, one FP64 atomic each
     // (Bellman-Ford's counts in FP32: only a zero matters, and no sum rounds to it)
@@ -294,7 +299,8 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
     for (int c = tid; c < S; c += NT) {
         if constexpr (!BF) {
             s_T[c] = c < B ? (sync ? 1.0 : (double)p.g_coef) * ld_relaxed_f64(&p.T[c]) : 0.0;
-            s_g[c] = sync && c < B ? ld_relaxed_f64(&p.acc_g[2 * B + c]) : 0.0;
+            s_live[c] = 0.0;
+            s_gt[c] = c < B ? dangling(ld_relaxed_f64(&p.acc_g[2 * B + c]), s_T[c]) : 0.0f;
         }
         s_last[c] = 0;
         s_run[c] = c < B ? 1 : 0;
@@ -324,7 +330,7 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
                 xo[q][e] = 0u;
                 if (has(q)) {
                     act[q] |= s_run[col0(q) + e] ? 1u << e : 0u;
-                    if (!BF && sync) gt[q][e] = (float)((double)p.g_coef * (s_T[col0(q) + e] - s_g[col0(q) + e]));
+                    if (!BF) gt[q][e] = s_gt[col0(q) + e];
                 }
             }
         }
@@ -337,26 +343,24 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
             for (int q = 0; q < CH; ++q)
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    if (mass[q][e] != 0.0f) atomicAdd(&s_g[col0(q) + e], (double)mass[q][e]);
+                    if (mass[q][e] != 0.0f) atomicAdd(&s_live[col0(q) + e], (double)mass[q][e]);
                     mass[q][e] = 0.0f;
                 }
         };
-        auto live = [&](bool first) {
-            if (!first) {
-                give_mass();
-                if ((++turn & (RUN_WARPS - 1)) == 0)
-                    for (int c = lane; c < B; c += 32) {
-                        const double v = __longlong_as_double((long long)atomicExch((unsigned long long*)&s_g[c], 0ULL));
-                        if (v != 0.0) atomicAdd(&p.gl[c], v);
-                    }
-            }
+        auto live = [&]() {
+            give_mass();
+            if ((++turn & (RUN_WARPS - 1)) == 0)
+                for (int c = lane; c < B; c += 32) {
+                    const double v = __longlong_as_double((long long)atomicExch((unsigned long long*)&s_live[c], 0ULL));
+                    if (v != 0.0) atomicAdd(&p.gl[c], v);
+                }
 #pragma unroll
             for (int q = 0; q < CH; ++q)
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     if (!((act[q] >> e) & 1u)) continue;
                     const int c = col0(q) + e;
-                    gt[q][e] = (float)fma(-(double)p.g_coef, ld_relaxed_f64(&p.gl[c]), s_T[c]);
+                    gt[q][e] = dangling(ld_relaxed_f64(&p.gl[c]), s_T[c]);
                 }
         };
         // row v's new values from its sum (every group holds it) and inputs; group 0 stores them
@@ -511,7 +515,6 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
             }
         };
         load_raw();
-        if (!BF && !sync && t == w) live(true);  // (while the first loads of the sweep are in flight)
         // The next items of the run into list half lb (all of them, or for Bellman-Ford the ones a sweep needs);
         // an empty stage means that the run is done.
         auto build = [&](int lb) -> RunStage {
@@ -748,7 +751,7 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
                 half = (half + ncb) & 1;
                 lb ^= 1;
                 fb -= ncb;
-                if (!BF && !sync && (++stages & (LIVE_STAGES - 1)) == 0) live(false);
+                if (!BF && !sync && (++stages & (LIVE_STAGES - 1)) == 0) live();
             }
         }
 
@@ -791,16 +794,20 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
         if (!BF) cta_sum(mass, sync ? p.acc_g + slot * B : p.gl, nullptr);
         if (!BF && !sync)  // what the warps gave during the sweep (cta_sum's barriers stand before and after)
             for (int c = tid; c < B; c += NT) {
-                const double v = s_g[c];
+                const double v = s_live[c];
                 if (v != 0.0) atomicAdd(&p.gl[c], v);
-                s_g[c] = 0.0;
+                s_live[c] = 0.0;
             }
         if (!grid_barrier(p.sb, p.nblocks, bar, p.timeout_ns)) return;
         int still = 0;
         for (int c = tid; c < B; c += NT) {
-            if (!BF && sync) s_g[c] = ld_relaxed_f64(&p.acc_g[slot * B + c]);
+            // the sweep's first dangling term for the whole CTA: while every warp read the live mass at its first run, the
+            // columns' few lines in L2 held up small graphs (PPR of 32 columns, uniform, 3 K vertices 200 -> 146 us, 30 K
+            // 395 -> 342; synchronous, formed per lane before, 169 -> 146; 256 columns at 1 M vertices the same)
+            const double res = ld_relaxed_f64(&p.acc_res[slot * B + c]);
+            if (!BF) s_gt[c] = dangling(ld_relaxed_f64(sync ? &p.acc_g[slot * B + c] : &p.gl[c]), s_T[c]);
             if (s_run[c]) {
-                if (ld_relaxed_f64(&p.acc_res[slot * B + c]) <= p.tol) {
+                if (res <= p.tol) {
                     s_run[c] = 0;
                     s_last[c] = it + 1;
                     if (blockIdx.x == 0) p.iters[c] = it + 1;
@@ -880,7 +887,7 @@ size_t run_smem_bytes(bool is_bf, int B)
     const size_t S = (size_t)((B + 3) & ~3);
     const int k = run_shape(B), depth = run_depth(k < 5 ? 1 << k : 32, k > 5 ? 1 << (k - 5) : 1);
     const size_t SR = run_padded(is_bf, k < 5 ? 1 << k : 32, k > 5 ? 1 << (k - 5) : 1) ? (size_t)4 << k : S;
-    return (is_bf ? 0 : 2 * S * 8) + 2 * RUN_WARPS * S * 4 + 2 * S * 4 + RUN_WARPS * 128 * 4 +
+    return (is_bf ? 0 : 2 * S * 8 + S * 4) + 2 * RUN_WARPS * S * 4 + 2 * S * 4 + RUN_WARPS * 128 * 4 +
            (size_t)RUN_WARPS * depth * SR * 4;
 }
 
