@@ -621,9 +621,10 @@ static const void* warp_kernel(int kind, int mode, int variant, int ipt, bool or
 // 1.95 + 1.79, 1.99 + 1.98. Bellman-Ford on warp runs, whose edges cost more (a weight each) and rows less (no degree),
 // RMAT, 4 M vertices, four-byte weights, 224-item tiles, weights 1, 2, 3: sync 4.34, 3.91, 3.97, delta 16 4.03, 3.83, 3.60,
 // delta 256 with cached reads 4.41, 3.95, 4.36, async 3.88, 3.45, 3.48; one-byte weights the same order, 2 to 5% less. Graphs
-// without skew do not move. (The tiles' merge-path walk over runs of equal item counts, in the same order: 3.71, 3.51, 4.07,
-// 3.46. Synchronous Bellman-Ford on 224-item tiles is the form that lost by the change, 5% at 4 M and 2 M RMAT vertices; it
-// gained 9% at 1 M, 11% with 160-item tiles at 4 M, 7 to 24% on uniform and banded graphs.)
+// without skew do not move. (Each figure is of one plan: where a plan's arrays land in memory moves RMAT's solves by up to
+// 9%. Over ten placements, 4 M vertices, four-byte weights, us a sweep, against the tiles' merge-path walk over runs of
+// equal item counts: sync 265.5 and 265.3, delta 16 284 and 293, delta 256 cached 300 and 293, async 282 and 291; 1 M 5 to
+// 8% less but delta 256 1% more, uniform and banded graphs 4 to 26% less.)
 static int warp_row_weight(int kind, int mode)
 {
     return kind == WARP_RUNS && (mode == MODE_BF || mode == MODE_BF8) ? 2 : 3;
