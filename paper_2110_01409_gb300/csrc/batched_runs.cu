@@ -117,9 +117,9 @@ constexpr unsigned PUB_EMPTY = 1u;   // the published partial is the identity: i
 constexpr int FOLD_STAGES = 2;       // PPR: stages inside one row after which its sum is folded
 constexpr int LIVE_STAGES = 16;      // asynchronous PPR: a warp adds to and reads the live mass every 16 stages
 
-// Up to 32 items of a run, in order, as the fetches they need. Vertex and weight (PPR: the row's out-degree) of
-// item k are in the warp's list; `old` marks the items that read a row's old values, `fin` the row's last item (PPR: its teleport
-// entries; Bellman-Ford: the old values themselves).
+// Up to 32 items of a run, in order, as the fetches they need. Vertex and weight (PPR: the row's out-degree) of item k
+// are in the warp's list; `old` marks the items that read a row's old values, `fin` the row's last item (PPR: its
+// teleport entries; Bellman-Ford: the old values themselves).
 struct RunStage {
     unsigned old, fin;
     int cnt;
@@ -492,224 +492,224 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
         int pend = -1, pend_row = 0;  // the run whose first row waits for earlier runs' partials
         bool ok = true;
         for (int t = w; t < p.nruns && ok; t += W) {
-        // ---------------- run t, as a stream of fetches ----------------
-        // rows [i0, i_end) end in this run; head: it starts inside row i0 and ends it
-        const int i0 = t == w ? first_i0 : p.run_row[t], i_end = t == w ? first_ie : p.run_row[t + 1];
-        const int j0 = t == w ? first_j0 : p.run_nz[t], j_end = t == w ? first_je : p.run_nz[t + 1];
-        const bool head = t == w ? first_head : j0 > p.rowptr[i0] && i_end > i0;
-        int i = i0, j = j0, ph = 0;   // next row end, next in-edge, 1: row i's old values are behind, its V ahead
-        bool carry_need = false;      // BF: the row in progress has a kept in-edge in an earlier stage
-        bool head_pending = head;
-        int whole = 0;                // PPR: stages in a row that ended no row (a long row's sum is folded, below)
-        bool folded = false;
-        // the next stage's row ends and in-edges, loaded while the current one is walked
-        int raw_end, raw_col;
-        uint32_t raw_w = 0u;  // BF: the in-edges' weights; PPR: the rows' out-degrees (float bits)
-        auto load_raw = [&]() {
-            raw_end = i + lane < i_end ? ld_stream_i32(p.rowptr + i + lane + 1) : INT_MAX;
-            raw_col = 0;
-            if constexpr (!BF) raw_w = i + lane < i_end ? __float_as_uint(ld_stream_f32(p.degf + i + lane)) : 0u;
-            if (j + lane < j_end) {
-                raw_col = ld_stream_i32(p.colidx + j + lane);
-                if constexpr (BF) raw_w = p.w8 ? (uint32_t)p.w8[j + lane] : ld_stream_u32(p.w + j + lane);
-            }
-        };
-        load_raw();
-        // The next items of the run into list half lb (all of them, or for Bellman-Ford the ones a sweep needs);
-        // an empty stage means that the run is done.
-        auto build = [&](int lb) -> RunStage {
-            RunStage st{0u, 0u, 0};
-            int* lv = list + lb * 64;
-            for (;;) {
-                const int left = (j_end - j) + RW * (i_end - i) - ph;
-                const int cnt = min(32, left);
-                if (cnt <= 0) return st;
-                const int pos = raw_end == INT_MAX ? INT_MAX : (raw_end - j) + RW * lane - ph;  // of row i + lane's old
-                unsigned old = __reduce_or_sync(FULL, (pos >= 0 && pos < cnt) ? 1u << pos : 0u);
-                unsigned fin = old;
-                if constexpr (!BF)
-                    fin = __reduce_or_sync(FULL, (pos != INT_MAX && pos + 1 >= 0 && pos + 1 < cnt) ? 1u << (pos + 1) : 0u);
-                const unsigned special = old | fin;
-                const int eo = lane - __popc(special & below(lane));  // in-edge of item `lane`, from j
-                const int row = i + __popc(fin & below(lane));
-                const int src = __shfl_sync(FULL, raw_col, eo & 31);
-                const uint32_t wt = __shfl_sync(FULL, raw_w, (BF ? eo : row - i) & 31);
-                const bool sp = (special >> lane) & 1u;
-                const int vert = sp ? row : src;
-                int kept = cnt;
-                if constexpr (BF) {
-                    // in-edges whose source changed in this sweep or the one before; rows that keep any, the run's
-                    // first row while earlier runs hold a part of it, and (synchronous) rows whose other buffer is
-                    // a sweep behind
-                    const unsigned c = lane < cnt && (!sp || sync) ? p.chg[vert] : 128u;
-                    const bool fresh = lane < cnt && !sp && (c == now || c == before);
-                    const unsigned edges = __ballot_sync(FULL, fresh);
-                    const unsigned prior = special & below(lane);
-                    const int from = prior ? 32 - __clz(prior) : 0;
-                    const bool any = (edges & below(lane) & ~below(from)) != 0u || (!prior && carry_need);
-                    const bool keep_row = lane < cnt && sp && (any || (head && row == i0) || (sync && c == before));
-                    const unsigned need = edges | __ballot_sync(FULL, keep_row);
-                    const int last = special & below(cnt) ? 32 - __clz(special & below(cnt)) : 0;
-                    carry_need = (edges & ~below(last)) != 0u || (last == 0 && carry_need);
-                    kept = __popc(need);
-                    const int at = __popc(need & below(lane));
-                    old = fin = __reduce_or_sync(FULL, keep_row ? 1u << at : 0u);
-                    if ((need >> lane) & 1u) {
-                        lv[at] = vert;
-                        lv[32 + at] = (int)wt;
-                    }
-                } else {
-                    if (lane < cnt) {
-                        lv[lane] = vert;
-                        lv[32 + lane] = (int)wt;
-                    }
-                }
-                const unsigned all = special & below(cnt);
-                const int ended = __popc(BF ? all : fin);
-                ph = (!BF && ((old >> (cnt - 1)) & 1u)) ? 1 : 0;  // the old values were the stage's last item
-                i += ended;
-                j += cnt - __popc(all);
-                load_raw();
-                if (kept > 0) {
-                    st.old = old;
-                    st.fin = fin;
-                    st.cnt = kept;
-                    __syncwarp();
-                    return st;
-                }
-            }
-        };
-        auto fold_in = [&](uint32_t (&a)[CH][4]) {  // the groups' joined part of the row in progress
-#pragma unroll
-            for (int q = 0; q < CH; ++q)
-                if (has(q))
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        if (grp == 0) fold[col0(q) + e] = folded ? comb<BF>(fold[col0(q) + e], a[q][e]) : a[q][e];
-                        a[q][e] = ident<BF>();
-                    }
-            folded = true;
-            __syncwarp();
-        };
-        auto unfold = [&](uint32_t (&a)[CH][4]) {  // adds it back, in every group
-#pragma unroll
-            for (int q = 0; q < CH; ++q)
-                if (has(q))
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) a[q][e] = comb<BF>(a[q][e], fold[col0(q) + e]);
-            folded = false;
-            __syncwarp();
-        };
-        auto batches = [&](const RunStage& st) { return (st.cnt + G - 1) / G; };
-        constexpr int STEPS = G >= GRP ? G / GRP : 1;  // groups' turns in a batch
-        // copies of batch b of a stage into ring half `half`
-        auto fetch = [&](const RunStage& st, int lb, int b, int half) {
-            const int* lv = list + lb * 64 + b * G;
-            const uint32_t at = ring_at + (uint32_t)(half * G * SR + 4 * lr) * 4u;
-            const int have = st.cnt - b * G;
-            const unsigned tele = BF ? 0u : st.fin >> (b * G);
-#pragma unroll
-            for (int u = 0; u < STEPS; ++u) {
-                const int k = u * GRP + grp;
-                if (k >= have || (G < GRP && k >= G)) continue;
-                const int v = lv[k];
-                const uint32_t dst = at + (uint32_t)(k * SR) * 4u;
-                if (BF || !((tele >> k) & 1u)) {
-                    const uint32_t* x = xin + (size_t)v * S;
-#pragma unroll
-                    for (int q = 0; q < CH; ++q)
-                        if (EVERY || has(q)) cp16(dst + 512u * q, x + from(q));
-                } else if (p.v16) {
-                    const float* x = p.V + (size_t)v * B;
-#pragma unroll
-                    for (int q = 0; q < CH; ++q)
-                        if (EVERY || has(q)) cp16(dst + 512u * q, x + from(q));
-                } else {
-#pragma unroll
-                    for (int q = 0; q < CH; ++q)
-#pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            if (has(q) && col0(q) + e < B)
-                                cp4(dst + 512u * q + 4u * e, p.V + (size_t)v * B + col0(q) + e);
-                }
-            }
-        };
-        // batch b of a stage from ring half `half`
-        auto consume = [&](const RunStage& st, int lb, int b, int half) {
-            const int* lv = list + lb * 64 + b * G;
-            const uint32_t* rows = ring + half * G * SR + 4 * lr;
-            auto add = [&](int k) {
-                const uint32_t wt = BF ? (uint32_t)lv[32 + k] : 0u;
-#pragma unroll
-                for (int q = 0; q < CH; ++q) {
-                    if (!PAD && !has(q)) continue;
-                    const uint4 x = *(const uint4*)(rows + k * SR + 128 * q);
-                    acc[q][0] = comb<BF>(acc[q][0], BF ? relax_w(x.x, wt) : x.x);
-                    acc[q][1] = comb<BF>(acc[q][1], BF ? relax_w(x.y, wt) : x.y);
-                    acc[q][2] = comb<BF>(acc[q][2], BF ? relax_w(x.z, wt) : x.z);
-                    acc[q][3] = comb<BF>(acc[q][3], BF ? relax_w(x.w, wt) : x.w);
+            // ---------------- run t, as a stream of fetches ----------------
+            // rows [i0, i_end) end in this run; head: it starts inside row i0 and ends it
+            const int i0 = t == w ? first_i0 : p.run_row[t], i_end = t == w ? first_ie : p.run_row[t + 1];
+            const int j0 = t == w ? first_j0 : p.run_nz[t], j_end = t == w ? first_je : p.run_nz[t + 1];
+            const bool head = t == w ? first_head : j0 > p.rowptr[i0] && i_end > i0;
+            int i = i0, j = j0, ph = 0;   // next row end, next in-edge, 1: row i's old values are behind, its V ahead
+            bool carry_need = false;      // BF: the row in progress has a kept in-edge in an earlier stage
+            bool head_pending = head;
+            int whole = 0;                // PPR: stages in a row that ended no row (a long row's sum is folded, below)
+            bool folded = false;
+            // the next stage's row ends and in-edges, loaded while the current one is walked
+            int raw_end, raw_col;
+            uint32_t raw_w = 0u;  // BF: the in-edges' weights; PPR: the rows' out-degrees (float bits)
+            auto load_raw = [&]() {
+                raw_end = i + lane < i_end ? ld_stream_i32(p.rowptr + i + lane + 1) : INT_MAX;
+                raw_col = 0;
+                if constexpr (!BF) raw_w = i + lane < i_end ? __float_as_uint(ld_stream_f32(p.degf + i + lane)) : 0u;
+                if (j + lane < j_end) {
+                    raw_col = ld_stream_i32(p.colidx + j + lane);
+                    if constexpr (BF) raw_w = p.w8 ? (uint32_t)p.w8[j + lane] : ld_stream_u32(p.w + j + lane);
                 }
             };
-            const int have = min(G, st.cnt - b * G);
-            unsigned rem = ((st.old | st.fin) >> (b * G)) & below(have);
-            if (rem == 0u) {  // in-edges only
+            load_raw();
+            // The next items of the run into list half lb (all of them, or for Bellman-Ford the ones a sweep needs);
+            // an empty stage means that the run is done.
+            auto build = [&](int lb) -> RunStage {
+                RunStage st{0u, 0u, 0};
+                int* lv = list + lb * 64;
+                for (;;) {
+                    const int left = (j_end - j) + RW * (i_end - i) - ph;
+                    const int cnt = min(32, left);
+                    if (cnt <= 0) return st;
+                    const int pos = raw_end == INT_MAX ? INT_MAX : (raw_end - j) + RW * lane - ph;  // of row i + lane's old
+                    unsigned old = __reduce_or_sync(FULL, (pos >= 0 && pos < cnt) ? 1u << pos : 0u);
+                    unsigned fin = old;
+                    if constexpr (!BF)
+                        fin = __reduce_or_sync(
+                            FULL, (pos != INT_MAX && pos + 1 >= 0 && pos + 1 < cnt) ? 1u << (pos + 1) : 0u);
+                    const unsigned special = old | fin;
+                    const int eo = lane - __popc(special & below(lane));  // in-edge of item `lane`, from j
+                    const int row = i + __popc(fin & below(lane));
+                    const int src = __shfl_sync(FULL, raw_col, eo & 31);
+                    const uint32_t wt = __shfl_sync(FULL, raw_w, (BF ? eo : row - i) & 31);
+                    const bool sp = (special >> lane) & 1u;
+                    const int vert = sp ? row : src;
+                    int kept = cnt;
+                    if constexpr (BF) {
+                        // in-edges whose source changed in this sweep or the one before; rows that keep any, the run's
+                        // first row while earlier runs hold a part of it, and (synchronous) rows whose other buffer is
+                        // a sweep behind
+                        const unsigned c = lane < cnt && (!sp || sync) ? p.chg[vert] : 128u;
+                        const bool fresh = lane < cnt && !sp && (c == now || c == before);
+                        const unsigned edges = __ballot_sync(FULL, fresh);
+                        const unsigned prior = special & below(lane);
+                        const int from = prior ? 32 - __clz(prior) : 0;
+                        const bool any = (edges & below(lane) & ~below(from)) != 0u || (!prior && carry_need);
+                        const bool keep_row = lane < cnt && sp && (any || (head && row == i0) || (sync && c == before));
+                        const unsigned need = edges | __ballot_sync(FULL, keep_row);
+                        const int last = special & below(cnt) ? 32 - __clz(special & below(cnt)) : 0;
+                        carry_need = (edges & ~below(last)) != 0u || (last == 0 && carry_need);
+                        kept = __popc(need);
+                        const int at = __popc(need & below(lane));
+                        old = fin = __reduce_or_sync(FULL, keep_row ? 1u << at : 0u);
+                        if ((need >> lane) & 1u) {
+                            lv[at] = vert;
+                            lv[32 + at] = (int)wt;
+                        }
+                    } else {
+                        if (lane < cnt) {
+                            lv[lane] = vert;
+                            lv[32 + lane] = (int)wt;
+                        }
+                    }
+                    const unsigned all = special & below(cnt);
+                    const int ended = __popc(BF ? all : fin);
+                    ph = (!BF && ((old >> (cnt - 1)) & 1u)) ? 1 : 0;  // the old values were the stage's last item
+                    i += ended;
+                    j += cnt - __popc(all);
+                    load_raw();
+                    if (kept > 0) {
+                        st.old = old;
+                        st.fin = fin;
+                        st.cnt = kept;
+                        __syncwarp();
+                        return st;
+                    }
+                }
+            };
+            auto fold_in = [&](uint32_t (&a)[CH][4]) {  // the groups' joined part of the row in progress
+#pragma unroll
+                for (int q = 0; q < CH; ++q)
+                    if (has(q))
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            if (grp == 0) fold[col0(q) + e] = folded ? comb<BF>(fold[col0(q) + e], a[q][e]) : a[q][e];
+                            a[q][e] = ident<BF>();
+                        }
+                folded = true;
+                __syncwarp();
+            };
+            auto unfold = [&](uint32_t (&a)[CH][4]) {  // adds it back, in every group
+#pragma unroll
+                for (int q = 0; q < CH; ++q)
+                    if (has(q))
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) a[q][e] = comb<BF>(a[q][e], fold[col0(q) + e]);
+                folded = false;
+                __syncwarp();
+            };
+            auto batches = [&](const RunStage& st) { return (st.cnt + G - 1) / G; };
+            constexpr int STEPS = G >= GRP ? G / GRP : 1;  // groups' turns in a batch
+            // copies of batch b of a stage into ring half `half`
+            auto fetch = [&](const RunStage& st, int lb, int b, int half) {
+                const int* lv = list + lb * 64 + b * G;
+                const uint32_t at = ring_at + (uint32_t)(half * G * SR + 4 * lr) * 4u;
+                const int have = st.cnt - b * G;
+                const unsigned tele = BF ? 0u : st.fin >> (b * G);
 #pragma unroll
                 for (int u = 0; u < STEPS; ++u) {
                     const int k = u * GRP + grp;
-                    if (k < have) add(k);
-                }
-                return;
-            }
-            const unsigned old = BF ? 0u : st.old >> (b * G);
-            int a = 0;
-            for (;;) {
-                const int e1 = rem ? __ffs(rem) - 1 : have;
-                for (int k = a + grp; k < e1; k += GRP) add(k);
-                if (!rem) break;
-                rem &= rem - 1u;
-                a = e1 + 1;
-                uint4 x[CH];
+                    if (k >= have || (G < GRP && k >= G)) continue;
+                    const int v = lv[k];
+                    const uint32_t dst = at + (uint32_t)(k * SR) * 4u;
+                    if (BF || !((tele >> k) & 1u)) {
+                        const uint32_t* x = xin + (size_t)v * S;
 #pragma unroll
-                for (int q = 0; q < CH; ++q) {
-                    x[q] = make_uint4(0u, 0u, 0u, 0u);
-                    if (PAD || has(q)) x[q] = *(const uint4*)(rows + e1 * SR + 128 * q);
+                        for (int q = 0; q < CH; ++q)
+                            if (EVERY || has(q)) cp16(dst + 512u * q, x + from(q));
+                    } else if (p.v16) {
+                        const float* x = p.V + (size_t)v * B;
+#pragma unroll
+                        for (int q = 0; q < CH; ++q)
+                            if (EVERY || has(q)) cp16(dst + 512u * q, x + from(q));
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < CH; ++q)
+#pragma unroll
+                            for (int e = 0; e < 4; ++e)
+                                if (has(q) && col0(q) + e < B)
+                                    cp4(dst + 512u * q + 4u * e, p.V + (size_t)v * B + col0(q) + e);
+                    }
                 }
-                if (!BF && ((old >> e1) & 1u)) {
+            };
+            // batch b of a stage from ring half `half`
+            auto consume = [&](const RunStage& st, int lb, int b, int half) {
+                const int* lv = list + lb * 64 + b * G;
+                const uint32_t* rows = ring + half * G * SR + 4 * lr;
+                auto add = [&](int k) {
+                    const uint32_t wt = BF ? (uint32_t)lv[32 + k] : 0u;
 #pragma unroll
                     for (int q = 0; q < CH; ++q) {
-                        xo[q][0] = x[q].x; xo[q][1] = x[q].y; xo[q][2] = x[q].z; xo[q][3] = x[q].w;
+                        if (!PAD && !has(q)) continue;
+                        const uint4 x = *(const uint4*)(rows + k * SR + 128 * q);
+                        acc[q][0] = comb<BF>(acc[q][0], BF ? relax_w(x.x, wt) : x.x);
+                        acc[q][1] = comb<BF>(acc[q][1], BF ? relax_w(x.y, wt) : x.y);
+                        acc[q][2] = comb<BF>(acc[q][2], BF ? relax_w(x.z, wt) : x.z);
+                        acc[q][3] = comb<BF>(acc[q][3], BF ? relax_w(x.w, wt) : x.w);
                     }
-                    continue;
+                };
+                const int have = min(G, st.cnt - b * G);
+                unsigned rem = ((st.old | st.fin) >> (b * G)) & below(have);
+                if (rem == 0u) {  // in-edges only
+#pragma unroll
+                    for (int u = 0; u < STEPS; ++u) {
+                        const int k = u * GRP + grp;
+                        if (k < have) add(k);
+                    }
+                    return;
                 }
-                join_groups(acc);
-                if (!BF && folded) unfold(acc);
-                if (head_pending) {  // begun in an earlier run: finished after this one
+                const unsigned old = BF ? 0u : st.old >> (b * G);
+                int a = 0;
+                for (;;) {
+                    const int e1 = rem ? __ffs(rem) - 1 : have;
+                    for (int k = a + grp; k < e1; k += GRP) add(k);
+                    if (!rem) break;
+                    rem &= rem - 1u;
+                    a = e1 + 1;
+                    uint4 x[CH];
+#pragma unroll
+                    for (int q = 0; q < CH; ++q) {
+                        x[q] = make_uint4(0u, 0u, 0u, 0u);
+                        if (PAD || has(q)) x[q] = *(const uint4*)(rows + e1 * SR + 128 * q);
+                    }
+                    if (!BF && ((old >> e1) & 1u)) {
+#pragma unroll
+                        for (int q = 0; q < CH; ++q) {
+                            xo[q][0] = x[q].x; xo[q][1] = x[q].y; xo[q][2] = x[q].z; xo[q][3] = x[q].w;
+                        }
+                        continue;
+                    }
+                    join_groups(acc);
+                    if (!BF && folded) unfold(acc);
+                    if (head_pending) {  // begun in an earlier run: finished after this one
+#pragma unroll
+                        for (int q = 0; q < CH; ++q)
+                            if (grp == 0 && has(q))
+                                *(uint4*)(head_sum + col0(q)) = make_uint4(acc[q][0], acc[q][1], acc[q][2], acc[q][3]);
+                        head_pending = false;
+                    } else {
+                        float tv[CH][4];
+#pragma unroll
+                        for (int q = 0; q < CH; ++q) {
+                            if constexpr (BF) {
+                                xo[q][0] = x[q].x; xo[q][1] = x[q].y; xo[q][2] = x[q].z; xo[q][3] = x[q].w;
+                            } else {
+                                tv[q][0] = __uint_as_float(x[q].x); tv[q][1] = __uint_as_float(x[q].y);
+                                tv[q][2] = __uint_as_float(x[q].z); tv[q][3] = __uint_as_float(x[q].w);
+                            }
+                        }
+                        update(lv[e1], acc, xo, tv, BF ? 0.0f : __int_as_float(lv[32 + e1]));
+                    }
 #pragma unroll
                     for (int q = 0; q < CH; ++q)
-                        if (grp == 0 && has(q))
-                            *(uint4*)(head_sum + col0(q)) = make_uint4(acc[q][0], acc[q][1], acc[q][2], acc[q][3]);
-                    head_pending = false;
-                } else {
-                    float tv[CH][4];
 #pragma unroll
-                    for (int q = 0; q < CH; ++q) {
-                        if constexpr (BF) {
-                            xo[q][0] = x[q].x; xo[q][1] = x[q].y; xo[q][2] = x[q].z; xo[q][3] = x[q].w;
-                        } else {
-                            tv[q][0] = __uint_as_float(x[q].x); tv[q][1] = __uint_as_float(x[q].y);
-                            tv[q][2] = __uint_as_float(x[q].z); tv[q][3] = __uint_as_float(x[q].w);
-                        }
-                    }
-                    update(lv[e1], acc, xo, tv, BF ? 0.0f : __int_as_float(lv[32 + e1]));
+                        for (int e = 0; e < 4; ++e) acc[q][e] = ident<BF>();
                 }
-#pragma unroll
-                for (int q = 0; q < CH; ++q)
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) acc[q][e] = ident<BF>();
-            }
-        };
+            };
 
-            {
             int lb = 0, half = 0, fb = 0;  // list half and first ring half of `cur`; batches fetched, from cur's first
             RunStage cur = build(0), nxt{0u, 0u, 0};
             bool ahead = false;            // nxt is built
@@ -753,40 +753,39 @@ __global__ void __launch_bounds__(NT, run_min_blocks(BF, CH)) batched_runs_kerne
                 fb -= ncb;
                 if (!BF && !sync && (++stages & (LIVE_STAGES - 1)) == 0) live();
             }
-        }
 
-        // ---------------- the row this run leaves unfinished, and the one it started inside ----------------
-        join_groups(acc);
-        if (!BF && folded) unfold(acc);
-        bool some = false;
-#pragma unroll
-        for (int q = 0; q < CH; ++q)
-            if (has(q))
-#pragma unroll
-                for (int e = 0; e < 4; ++e) some |= acc[q][e] != ident<BF>();
-        some = __any_sync(FULL, some);
-        if (some && grp == 0) {
+            // ---------------- the row this run leaves unfinished, and the one it started inside ----------------
+            join_groups(acc);
+            if (!BF && folded) unfold(acc);
+            bool some = false;
 #pragma unroll
             for (int q = 0; q < CH; ++q)
-                if (has(q)) st_relaxed_v4(p.part + (size_t)t * S + col0(q), acc[q]);
-        }
-        if (some) fence_gpu();
-        __syncwarp();
-        if (lane == 0) st_pub(p.pub + t, ((unsigned long long)stamp << 32) | (some ? 0u : PUB_EMPTY));
-        // the pending row is finished a run later, by when the runs before it have published theirs (a run publishes
-        // before its warp waits for an older one, so the lowest pending run can always finish)
-        if (pend >= 0) ok = resolve(pend, pend_row);
-        pend = head ? t : -1;
-        pend_row = i0;
-        if (head && grp == 0) {
+                if (has(q))
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) some |= acc[q][e] != ident<BF>();
+            some = __any_sync(FULL, some);
+            if (some && grp == 0) {
+#pragma unroll
+                for (int q = 0; q < CH; ++q)
+                    if (has(q)) st_relaxed_v4(p.part + (size_t)t * S + col0(q), acc[q]);
+            }
+            if (some) fence_gpu();
+            __syncwarp();
+            if (lane == 0) st_pub(p.pub + t, ((unsigned long long)stamp << 32) | (some ? 0u : PUB_EMPTY));
+            // the pending row is finished a run later, by when the runs before it have published theirs (a run publishes
+            // before its warp waits for an older one, so the lowest pending run can always finish)
+            if (pend >= 0) ok = resolve(pend, pend_row);
+            pend = head ? t : -1;
+            pend_row = i0;
+            if (head && grp == 0) {
+#pragma unroll
+                for (int q = 0; q < CH; ++q)
+                    if (has(q)) *(uint4*)(head_part + col0(q)) = *(const uint4*)(head_sum + col0(q));
+            }
 #pragma unroll
             for (int q = 0; q < CH; ++q)
-                if (has(q)) *(uint4*)(head_part + col0(q)) = *(const uint4*)(head_sum + col0(q));
-        }
 #pragma unroll
-        for (int q = 0; q < CH; ++q)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) acc[q][e] = ident<BF>();
+                for (int e = 0; e < 4; ++e) acc[q][e] = ident<BF>();
         }  // runs
         if (ok && pend >= 0) resolve(pend, pend_row);
         // ---------------- end of sweep: per-column sums, barrier, stopping rules ----------------
